@@ -208,6 +208,33 @@ int pw_advect_adjoint(pw_dtype dtype, const void *u, const void *v, const void *
 int pw_fold_periodic_halo(pw_dtype dtype, void *field, const pw_dims *dims, void *stream);
 
 /*
+ * pw_euler_periodic -- one forward-Euler update of three periodic fields:
+ * ou = u + dt su (likewise v, w) on the interior, each product and sum rounded
+ * once, and the halo of ou filled from its own interior as
+ * pw_fill_periodic_halo would. Columns nx+2 .. width-1 (row padding) are copied
+ * from u, v, w; nx + 2 <= width <= sy. The halo and padding of su, sv, sw are
+ * not read. dtype selects the element size (PW_F32_SPLIT and PW_F32 = float,
+ * with dt rounded to float, else double). All nine fields share `dims`; the
+ * outputs may not overlap the inputs or each other. Errors: PW_ENULL,
+ * PW_EINVAL, PW_EALIAS, PW_ECUDA.
+ */
+int pw_euler_periodic(pw_dtype dtype, const void* u, const void* v, const void* w, const void* su, const void* sv,
+                      const void* sw, double dt, const pw_dims* dims, int width, void* ou, void* ov, void* ow,
+                      void* stream);
+
+/*
+ * pw_euler_periodic_adjoint -- transpose of pw_euler_periodic: given the
+ * gradients g1, g2, g3 over every cell of ou, ov, ow, gu = g1 with its halo
+ * folded into the interior and cleared (as pw_fold_periodic_halo does in
+ * place), the gradient over u, and gsu = dt gu, the gradient over su; likewise
+ * v and w. Padding columns below width are copied (gu) and scaled (gsu).
+ * Errors as pw_euler_periodic.
+ */
+int pw_euler_periodic_adjoint(pw_dtype dtype, const void* g1, const void* g2, const void* g3, double dt,
+                              const pw_dims* dims, int width, void* gu, void* gv, void* gw, void* gsu, void* gsv,
+                              void* gsw, void* stream);
+
+/*
  * pw_advect_host_chunked -- pw_advect on fields that live in (pinned) host
  * memory, with the transfers overlapped with the computation (the paper's
  * Sec. IV chunking of host<->device traffic, here in slabs of levels). The

@@ -65,12 +65,37 @@ class FillPeriodicHalo(torch.autograd.Function):
         return out, None, None
 
 
+class EulerStep(torch.autograd.Function):
+    """(u, v, w) -> (u, v, w) + dt * F(u, v, w) with periodic halos; the
+    backward folds the halos and adds the adjoint kernel's gradient to the
+    folded one in place."""
+
+    @staticmethod
+    def forward(ctx, u, v, w, coeffs, nx, ny, dt, mode):
+        s = pw._uninitialised_like(u, 3)  # only their interior is read again
+        pw.advect(u, v, w, coeffs, nx, ny, mode=mode, out=s)
+        ctx.save_for_backward(u, v, w)
+        ctx.coeffs, ctx.nx, ctx.ny, ctx.dt, ctx.mode = coeffs, nx, ny, dt, mode
+        return pw.euler_periodic((u, v, w), s, dt, nx, ny)
+
+    @staticmethod
+    def backward(ctx, *grads):
+        u, v, w = ctx.saved_tensors
+        grads = tuple(g.contiguous() for g in grads)
+        gf, gs = pw.euler_periodic_adjoint(grads, ctx.dt, ctx.nx, ctx.ny, u)
+        pw.advect_adjoint(u, v, w, ctx.coeffs, ctx.nx, ctx.ny, *gs, mode=_ADJ_MODE[ctx.mode], out=gf, accumulate=True)
+        return (*gf, None, None, None, None, None)
+
+
 def advect(u, v, w, coeffs, nx, ny, mode="f64"):
     return PWAdvect.apply(u, v, w, coeffs, nx, ny, mode)
 
 
 def euler_step(u, v, w, coeffs, nx, ny, dt, mode="f64"):
     """x <- x + dt * F(x) on the interior, then a periodic halo refill."""
+    if isinstance(dt, (int, float)) and all(t.is_contiguous() for t in (u, v, w)):
+        return EulerStep.apply(u, v, w, coeffs, nx, ny, dt, mode)
+    # a dt that is a tensor (it may carry a gradient), or views of larger buffers
     su, sv, sw = advect(u, v, w, coeffs, nx, ny, mode)
     return tuple(FillPeriodicHalo.apply(f + dt * s, nx, ny) for f, s in zip((u, v, w), (su, sv, sw)))
 

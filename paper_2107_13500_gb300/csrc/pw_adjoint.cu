@@ -271,6 +271,18 @@ __global__ void __launch_bounds__(kPNT, 3) adjoint_paired_kernel(const __grid_co
 
     for (int k = kb; k < ke && !abort; ++k) {
         const int rc = k - kb + 1;  // relative level of k
+        if (a.accumulate) {
+            if (act_a) {
+                prefetch_l2(gu + g);
+                prefetch_l2(gv + g);
+                prefetch_l2(gw + g);
+            }
+            if (act_b) {
+                prefetch_l2(gu + g + kPHalf);
+                prefetch_l2(gv + g + kPHalf);
+                prefetch_l2(gw + g + kPHalf);
+            }
+        }
         if (rc + 2 < nl) {
             bad |= !wait(rc + 2);
             adj_convert(base + ((rc + 2) % kPS) * PSh::STAGE_BYTES, slot(rc + 2), cslot(rc + 2), k + 2, x0, y0, a,

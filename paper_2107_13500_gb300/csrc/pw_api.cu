@@ -504,6 +504,58 @@ extern "C" int pw_fold_periodic_halo(pw_dtype dtype, void* field, const pw_dims*
     return PW_OK;
 }
 
+// ---------------------------------------------------------------- time step
+
+// Checks shared by pw_euler_periodic and its adjoint: ins[nin] are read, outs[nout] written.
+static int check_step(pw_dtype dtype, const pw_dims* dims, int width, const void* const* ins, int nin,
+                      void* const* outs, int nout, const char* who) {
+    if (!known_dtype(dtype)) return fail(PW_EINVAL, "%s: unknown dtype %d", who, (int)dtype);
+    const int es = elem_size(dtype);
+    int rc = check_dims(dims, es, who);
+    if (rc) return rc;
+    if (width < dims->nx + 2 || width > dims->sy)
+        return fail(PW_EINVAL, "%s: width (%d) must lie in [nx + 2, sy]", who, width);
+    for (int n = 0; n < nin; ++n)
+        if ((rc = check_ptr(ins[n], es, "an input", who))) return rc;
+    const long long ext = field_extent_bytes(*dims, es) + (long long)(width - dims->nx - 2) * es;
+    for (int o = 0; o < nout; ++o) {
+        if ((rc = check_ptr(outs[o], es, "an output", who))) return rc;
+        for (int n = 0; n < nin; ++n)
+            if (overlap(outs[o], ext, ins[n], ext)) return fail(PW_EALIAS, "%s: an output overlaps an input", who);
+        for (int n = 0; n < o; ++n)
+            if (overlap(outs[o], ext, outs[n], ext)) return fail(PW_EALIAS, "%s: outputs overlap", who);
+    }
+    return PW_OK;
+}
+
+extern "C" int pw_euler_periodic(pw_dtype dtype, const void* u, const void* v, const void* w, const void* su,
+                                 const void* sv, const void* sw, double dt, const pw_dims* dims, int width, void* ou,
+                                 void* ov, void* ow, void* stream) {
+    const char* who = "pw_euler_periodic";
+    const void* ins[6] = {u, v, w, su, sv, sw};
+    void* outs[3] = {ou, ov, ow};
+    const int rc = check_step(dtype, dims, width, ins, 6, outs, 3, who);
+    if (rc) return rc;
+    const cudaError_t e =
+        pw::launch_euler_periodic(false, elem_size(dtype), ins, ins + 3, dt, dims->nx, dims->ny, dims->nz, width,
+                                  dims->sy, dims->sz, outs, nullptr, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? PW_OK : cuda_fail(e, who);
+}
+
+extern "C" int pw_euler_periodic_adjoint(pw_dtype dtype, const void* g1, const void* g2, const void* g3, double dt,
+                                         const pw_dims* dims, int width, void* gu, void* gv, void* gw, void* gsu,
+                                         void* gsv, void* gsw, void* stream) {
+    const char* who = "pw_euler_periodic_adjoint";
+    const void* ins[3] = {g1, g2, g3};
+    void* outs[6] = {gu, gv, gw, gsu, gsv, gsw};
+    const int rc = check_step(dtype, dims, width, ins, 3, outs, 6, who);
+    if (rc) return rc;
+    const cudaError_t e =
+        pw::launch_euler_periodic(true, elem_size(dtype), ins, nullptr, dt, dims->nx, dims->ny, dims->nz, width,
+                                  dims->sy, dims->sz, outs, outs + 3, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? PW_OK : cuda_fail(e, who);
+}
+
 // ---------------------------------------------------------------- batches
 
 extern "C" size_t pw_batch_plan_bytes(int n) { return pw::batch_plan_bytes(n); }

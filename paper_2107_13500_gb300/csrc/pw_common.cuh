@@ -101,6 +101,12 @@ __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// Bring the line of a global address into L2 (a read-modify-write issues this
+// a step ahead, so that its load does not wait for DRAM).
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(__cvta_generic_to_global(p)));
+}
+
 // Order this thread's earlier generic-proxy accesses of shared memory
 // before later async-proxy (TMA) writes to it.
 __device__ __forceinline__ void fence_proxy_async_smem() {

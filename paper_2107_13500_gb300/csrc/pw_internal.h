@@ -300,6 +300,13 @@ cudaError_t launch_fold_halo(void* field, int elem_bytes, int nx, int ny, int nz
 cudaError_t launch_fill_halo(void* field, int elem_bytes, int nx, int ny, int nz, long long sy, long long sz,
                              cudaStream_t st);
 
+// adjoint = false: o3 = a3 + dt b3 with a periodic halo; true: o3 = a3 with the
+// halo folded into the interior (and cleared), p3 = dt o3. Three fields of one
+// layout, columns 0..width-1 of every row.
+cudaError_t launch_euler_periodic(bool adjoint, int elem_bytes, const void* const* a3, const void* const* b3,
+                                  double dt, int nx, int ny, int nz, int width, long long sy, long long sz,
+                                  void* const* o3, void* const* p3, cudaStream_t st);
+
 cudaError_t launch_split_field(const double* f, long long fsy, long long fsz, float* fp, long long psy,
                                long long psz, int nx, int ny, int nz, double* mean, cudaStream_t st);
 

@@ -120,6 +120,12 @@ def load_library(path: str | None = None):
         lib.pw_energy_budget.argtypes = [vp, vp, vp, ctypes.c_int, ctypes.POINTER(Dims), vp, vp, vp, ctypes.c_int,
                                          ctypes.POINTER(Dims), vp, vp, vp, vp, vp]
         lib.pw_energy_budget.restype = ctypes.c_int
+        lib.pw_euler_periodic.argtypes = [ctypes.c_int] + [vp] * 6 + [ctypes.c_double, ctypes.POINTER(Dims),
+                                                                      ctypes.c_int] + [vp] * 4
+        lib.pw_euler_periodic.restype = ctypes.c_int
+        lib.pw_euler_periodic_adjoint.argtypes = [ctypes.c_int] + [vp] * 3 + [ctypes.c_double, ctypes.POINTER(Dims),
+                                                                              ctypes.c_int] + [vp] * 7
+        lib.pw_euler_periodic_adjoint.restype = ctypes.c_int
         _lib = lib
         return lib
 
@@ -171,6 +177,22 @@ def field_like(t):
     """Zeroed tensor with t's shape, dtype, device and 16-byte phase."""
     es = t.element_size()
     return _aligned_zeros(tuple(t.shape), t.dtype, t.device, (t.data_ptr() % 16) // es)
+
+
+def _uninitialised_like(t, count=None):
+    """field_like(t) without the zeros, for calls that write every cell they
+    read later. With a count, that many fields of one allocation (scratch that
+    no caller sees)."""
+    import torch
+    es = t.element_size()
+    lead = (t.data_ptr() % 16) // es
+    n, per = t.numel(), 16 // es
+    pitch = -(-n // per) * per  # fields of one allocation share the 16-byte phase
+    flat = torch.empty(lead + n + ((count or 1) - 1) * pitch, dtype=t.dtype, device=t.device)
+    stride = (t.shape[1] * t.shape[2], t.shape[2], 1)
+    if count is None:
+        return flat.as_strided(t.shape, stride, lead)
+    return tuple(flat.as_strided(t.shape, stride, lead + q * pitch) for q in range(count))
 
 
 def field_from_numpy(a, nx, dtype=None, device="cuda", aligned=True):
@@ -510,6 +532,41 @@ def fold_periodic_halo(g, nx, ny, stream=None):
     _check(load_library().pw_fold_periodic_halo(dt, ctypes.c_void_p(g.data_ptr()), ctypes.byref(d),
                                                 _stream_handle(stream)))
     return g
+
+
+# ---------------------------------------------------------------- time step
+
+def _step_dims(like, fields, nx, ny):
+    """(library dtype, dims) of contiguous fields of one shape and dtype."""
+    import torch
+    for t in fields:
+        if t.shape != like.shape or t.dtype != like.dtype or not t.is_contiguous():
+            raise ValueError("the fields of a step must be contiguous and share shape and dtype")
+    return (PW_F32 if like.dtype == torch.float32 else PW_F64), dims_of(like, nx, ny)
+
+
+def euler_periodic(fields, tendencies, dt, nx, ny, stream=None):
+    """f + dt * s of three fields, with periodic halos, in new fields
+    (pw_euler_periodic)."""
+    dtype, d = _step_dims(fields[0], tuple(fields) + tuple(tendencies), nx, ny)
+    out = tuple(_uninitialised_like(f) for f in fields)
+    vp = ctypes.c_void_p
+    _check(load_library().pw_euler_periodic(dtype, *(vp(t.data_ptr()) for t in tuple(fields) + tuple(tendencies)),
+                                            float(dt), ctypes.byref(d), fields[0].shape[2],
+                                            *(vp(t.data_ptr()) for t in out), _stream_handle(stream)))
+    return out
+
+
+def euler_periodic_adjoint(grads, dt, nx, ny, like, stream=None):
+    """Transpose of euler_periodic: (gradients over f, gradients over s), in
+    new fields with the 16-byte phase of `like`."""
+    dtype, d = _step_dims(like, grads, nx, ny)
+    gf, gs = tuple(_uninitialised_like(like) for _ in grads), _uninitialised_like(like, len(grads))
+    vp = ctypes.c_void_p
+    _check(load_library().pw_euler_periodic_adjoint(dtype, *(vp(t.data_ptr()) for t in grads), float(dt),
+                                                    ctypes.byref(d), like.shape[2],
+                                                    *(vp(t.data_ptr()) for t in gf + gs), _stream_handle(stream)))
+    return gf, gs
 
 
 # ---------------------------------------------------------------- batches
