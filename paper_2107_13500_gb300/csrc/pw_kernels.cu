@@ -3,6 +3,7 @@
 // and the device status word. The forward kernels live in pw_f64.cu (native
 // FP64), pw_paired.cu (paired FP32) and pw_split.cu (FP32); the adjoint in
 // pw_adjoint.cu.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -458,35 +459,71 @@ cudaError_t launch_split_field(const double* f, long long fsy, long long fsz, fl
 
 // ---------------------------------------------------------------------------
 // Energy budget: per level, the interior sums of u su, v sv, w sw and of their
-// absolute values, in FP64 and in a fixed order (columns strided over the
-// threads, rows in order; then a fixed shuffle tree and the warps in order),
-// so the result does not depend on scheduling. One CTA per (level, field).
-// A second single-CTA launch weights the level sums by the cell masses and
-// adds them level by level.
+// absolute values, in FP64 and in a fixed order, so the result does not depend
+// on scheduling. A cluster of kBudgetCluster CTAs sums one (level, field):
+// CTA r the r-th equal band of rows, each thread its columns in row order,
+// then a fixed shuffle tree, the warps in order and the CTAs in order (through
+// distributed shared memory, so no scratch memory is needed). A second
+// single-CTA launch weights the level sums by the cell masses and adds them
+// level by level.
+//
+// Bound by the FP64 pipe (two lane operations per clock per SM): each element
+// costs two of them, a sum and a sum of magnitudes, both as FMAs that round
+// the exact product into the running sum (a product, a sum and a sum of
+// magnitudes took three). Float inputs are widened by integer operations; the
+// hardware conversion, which issues on the FP64 pipe, serves only subnormals,
+// infinities and NaN. One CTA per (level, field) left 192 CTAs of a 64-level
+// domain on 152 SMs, so some SMs had twice the work of others; with clusters
+// of 8 there are 1536. 512x512x64 FP64: 203 us (3.97 TB/s, FP64 pipe 89 %
+// busy), 476 us before; with the totals 210 us a call, 487 before.
 
-constexpr int kBudgetThreads = 512;
+constexpr int kBudgetThreads = 256, kBudgetCluster = 8, kBudgetRows = 4;
+
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x);
+    const unsigned e = (b >> 23) & 0xFFu;
+    if (e - 1u < 254u || (b << 1) == 0) return float_bits_to_double(x);
+    return (double)x;
+}
 
 template <typename TW, typename TS>
-__global__ void __launch_bounds__(kBudgetThreads)
+__global__ void __cluster_dims__(kBudgetCluster, 1, 1) __launch_bounds__(kBudgetThreads)
     energy_level_kernel(const TW* __restrict__ u, const TW* __restrict__ v, const TW* __restrict__ w, long long wsy,
                         long long wsz, const TS* __restrict__ su, const TS* __restrict__ sv,
                         const TS* __restrict__ sw, long long ssy, long long ssz, int nx, int ny, int nz,
                         double* __restrict__ level_sums) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
     __shared__ double part[2][kBudgetThreads / 32];
-    const int k = blockIdx.x, f = blockIdx.y;
+    __shared__ double cta_sum[2];
+    const int rank = (int)blockIdx.x, k = blockIdx.y, f = blockIdx.z;  // the cluster spans the grid's x
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const TW* a = f == 0 ? u : f == 1 ? v : w;
-    const TS* b = f == 0 ? su : f == 1 ? sv : sw;
-    a += (size_t)k * (size_t)wsz;
-    b += (size_t)k * (size_t)ssz;
+    const int j0 = 1 + (int)((long long)ny * rank / kBudgetCluster);
+    const int j1 = 1 + (int)((long long)ny * (rank + 1) / kBudgetCluster);
+    const TW* a = (f == 0 ? u : f == 1 ? v : w) + (size_t)k * (size_t)wsz + (size_t)j0 * (size_t)wsy;
+    const TS* b = (f == 0 ? su : f == 1 ? sv : sw) + (size_t)k * (size_t)ssz + (size_t)j0 * (size_t)ssy;
     double s = 0.0, t = 0.0;
-    const TW* ar = a + wsy;  // row j = 1; rows advance by adding the stride
-    const TS* br = b + ssy;
-    for (int j = 1; j <= ny; ++j, ar += wsy, br += ssy) {
+    // rows in groups whose loads are all in flight; rows advance by adding the stride
+    for (int j = j0; j < j1; j += kBudgetRows, a += kBudgetRows * wsy, b += kBudgetRows * ssy) {
         for (int i = 1 + tid; i <= nx; i += kBudgetThreads) {
-            const double p = (double)__ldg(ar + i) * (double)__ldg(br + i);
-            s += p;
-            t += fabs(p);
+            TW x[kBudgetRows];
+            TS y[kBudgetRows];
+            const TW* pa = a + i;
+            const TS* pb = b + i;
+#pragma unroll
+            for (int q = 0; q < kBudgetRows; ++q) {
+                x[q] = j + q < j1 ? __ldg(pa) : TW(0);
+                y[q] = j + q < j1 ? __ldg(pb) : TS(0);
+                pa += wsy;
+                pb += ssy;
+            }
+#pragma unroll
+            for (int q = 0; q < kBudgetRows; ++q) {
+                const double xd = widen(x[q]), yd = widen(y[q]);
+                s = __fma_rn(xd, yd, s);
+                t = __fma_rn(fabs(xd), fabs(yd), t);
+            }
         }
     }
 #pragma unroll
@@ -502,18 +539,34 @@ __global__ void __launch_bounds__(kBudgetThreads)
     if (tid < 2) {
         double r = 0.0;
         for (int q = 0; q < kBudgetThreads / 32; ++q) r += part[tid][q];
+        cta_sum[tid] = r;
+    }
+    cluster.sync();
+    if (rank == 0 && tid < 2) {
+        double r = 0.0;
+        for (int q = 0; q < kBudgetCluster; ++q) r += *cluster.map_shared_rank(&cta_sum[tid], q);
         level_sums[(size_t)k * 6 + f + 3 * tid] = r;
     }
+    cluster.sync();  // no CTA leaves while its sums may still be read
 }
 
-__global__ void energy_total_kernel(const double* __restrict__ level_sums, const double* __restrict__ wu,
-                                    const double* __restrict__ ww, int nz, double* __restrict__ totals) {
-    const int n = threadIdx.x;
-    if (n >= 6) return;
+// Totals: warp n adds column n of the level sums. Lane l holds level 32 m + l
+// of group m (its loads in flight together); the products are then added level
+// by level, as the single-thread loop over nz did, whose dependent loads took
+// most of its 12.7 us at 64 levels.
+__global__ void __launch_bounds__(192)
+    energy_total_kernel(const double* __restrict__ level_sums, const double* __restrict__ wu,
+                        const double* __restrict__ ww, int nz, double* __restrict__ totals) {
+    const int n = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const double* wt = (n % 3 == 2) ? ww : wu;
     double r = 0.0;
-    for (int k = 0; k < nz; ++k) r += wt[k] * level_sums[(size_t)k * 6 + n];
-    totals[n] = r;
+    for (int k0 = 0; k0 < nz; k0 += 32) {
+        const int k = k0 + lane;
+        const double x = k < nz ? wt[k] : 0.0, y = k < nz ? level_sums[(size_t)k * 6 + n] : 0.0;
+        const int m = min(32, nz - k0);
+        for (int q = 0; q < m; ++q) r += __shfl_sync(0xffffffffu, x, q) * __shfl_sync(0xffffffffu, y, q);
+    }
+    if (lane == 0) totals[n] = r;
 }
 
 template <typename TW, typename TS>
@@ -521,13 +574,13 @@ static cudaError_t launch_energy_t(const void* u, const void* v, const void* w, 
                                    const void* su, const void* sv, const void* sw, long long ssy, long long ssz,
                                    int nx, int ny, int nz, const double* wu, const double* ww, double* level_sums,
                                    double* totals, cudaStream_t st) {
-    energy_level_kernel<TW, TS><<<dim3((unsigned)nz, 3), kBudgetThreads, 0, st>>>(
+    energy_level_kernel<TW, TS><<<dim3(kBudgetCluster, (unsigned)nz, 3), kBudgetThreads, 0, st>>>(
         static_cast<const TW*>(u), static_cast<const TW*>(v), static_cast<const TW*>(w), wsy, wsz,
         static_cast<const TS*>(su), static_cast<const TS*>(sv), static_cast<const TS*>(sw), ssy, ssz, nx, ny, nz,
         level_sums);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    energy_total_kernel<<<1, 32, 0, st>>>(level_sums, wu, ww, nz, totals);
+    energy_total_kernel<<<1, 192, 0, st>>>(level_sums, wu, ww, nz, totals);
     return cudaGetLastError();
 }
 
