@@ -134,7 +134,8 @@ int pw_fill_periodic_halo(pw_dtype dtype, void *field, const pw_dims *dims, void
  *   arrays in `c` are then not read, but c must still be non-NULL).
  * dtype PW_F32: u, v, w, su, sv, sw are float full fields; `split` is the
  *   table of pw_make_split_table built with all means 0 (it then carries
- *   only the coefficients, rounded to float).
+ *   only the coefficients, rounded to float; nothing else of it is read).
+ *   A table with means belongs to PW_F32_SPLIT, whichever fields it is for.
  * Errors: PW_ENULL, PW_EINVAL, PW_EALIAS, PW_EUNSUPPORTED, PW_ECUDA.
  */
 int pw_advect(pw_dtype dtype, const void *u, const void *v, const void *w, const pw_coeffs *c,

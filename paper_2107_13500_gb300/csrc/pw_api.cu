@@ -315,7 +315,7 @@ static int advect_levels(pw_dtype dtype, const void* u, const void* v, const voi
     switch (dtype) {
         case PW_F64: e = pw::launch_fwd_f64(mu, mv, mw, a, st); break;
         case PW_F64_PAIRED: e = pw::launch_fwd_paired(mu, mv, mw, a, st); break;
-        default: e = pw::launch_fwd_split(mu, mv, mw, a, st); break;
+        default: e = pw::launch_fwd_split(dtype == PW_F32, mu, mv, mw, a, st); break;
     }
     if (e != cudaSuccess) return cuda_fail(e, who);
     return PW_OK;
@@ -672,7 +672,7 @@ extern "C" int pw_advect_batched(pw_dtype dtype, int variant, void* plan_dev, lo
     if (e != cudaSuccess) return cuda_fail(e, who);
     e = dtype == PW_F64_PAIRED ? pw::launch_paired_batched(variant, plan, n_items, st)
         : dtype == PW_F64      ? pw::launch_f64_batched(variant, plan, n_items, st)
-                               : pw::launch_split_batched(variant, plan, n_items, st);
+                               : pw::launch_split_batched(dtype == PW_F32, variant, plan, n_items, st);
     if (e != cudaSuccess) return cuda_fail(e, who);
     return PW_OK;
 }

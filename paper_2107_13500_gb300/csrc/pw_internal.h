@@ -258,9 +258,8 @@ TileShape fwd_f64_shape_variant(int v);
 cudaError_t launch_f64_batched(int v, BatchPlan* plan, long long n_items, cudaStream_t st);
 int split_variant_count();
 TileShape fwd_split_shape_variant(int v);
-cudaError_t launch_fwd_split_variant(int v, const CUtensorMap& mu, const CUtensorMap& mv, const CUtensorMap& mw,
-                                     const FwdArgs& a, cudaStream_t st);
-cudaError_t launch_split_batched(int v, BatchPlan* plan, long long n_items, cudaStream_t st);
+// full: PW_F32 (full float fields), else PW_F32_SPLIT
+cudaError_t launch_split_batched(bool full, int v, BatchPlan* plan, long long n_items, cudaStream_t st);
 int paired_variant_count();
 TileShape fwd_paired_shape_variant(int v);
 cudaError_t launch_paired_batched(int v, BatchPlan* plan, long long n_items, cudaStream_t st);
@@ -269,7 +268,7 @@ cudaError_t launch_fwd_f64(const CUtensorMap& mu, const CUtensorMap& mv, const C
                            const FwdArgs& a, cudaStream_t st);
 cudaError_t launch_fwd_paired(const CUtensorMap& mu, const CUtensorMap& mv, const CUtensorMap& mw,
                               const FwdArgs& a, cudaStream_t st);
-cudaError_t launch_fwd_split(const CUtensorMap& mu, const CUtensorMap& mv, const CUtensorMap& mw,
+cudaError_t launch_fwd_split(bool full, const CUtensorMap& mu, const CUtensorMap& mv, const CUtensorMap& mw,
                              const FwdArgs& a, cudaStream_t st);
 
 struct AdjArgs {

@@ -94,7 +94,7 @@ extern "C" int pw_advect_batched_noalloc(pw_dtype dtype, int variant, const void
     if (e == cudaSuccess) e = cudaMemsetAsync(&plan->counter, 0, sizeof(plan->counter), st);
     if (e != cudaSuccess) return fail(PW_ECUDA, "pw_advect_batched_noalloc: copying the plan failed");
     e = dtype == PW_F64_PAIRED ? pw::launch_paired_batched(variant, plan, n_items, st)
-                               : pw::launch_split_batched(variant, plan, n_items, st);
+                               : pw::launch_split_batched(dtype == PW_F32, variant, plan, n_items, st);
     if (e != cudaSuccess) return fail(PW_ECUDA, "pw_advect_batched_noalloc: launch failed");
     return PW_OK;
 }

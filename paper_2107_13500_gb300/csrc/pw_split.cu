@@ -1,6 +1,6 @@
 // pw_split.cu -- PW advection in FP32 on perturbations about per-level FP64
-// means (PW_F32_SPLIT), and on full float fields (PW_F32 = the same kernel
-// with every mean 0).
+// means (PW_F32_SPLIT), and on full float fields (PW_F32 = the same march
+// with every mean 0, the mean terms left out).
 //
 // Writing u = U(k) + u' (likewise v, w) with U(k) the level mean, the mean x
 // mean parts of every horizontal flux difference cancel exactly, and each
@@ -34,6 +34,9 @@ constexpr int kRowBytes = PW_SPLIT_NCOEF * 4;
 // Resident warps per SM the one-shot and the persistent kernels are
 // compiled for, whatever the CTA size (the register budget follows).
 constexpr int kWarpsOneShot = 20, kWarpsBatched = 16;
+// The same for PW_F32, which needs fewer registers in the persistent kernel
+// (more than 20 warps spill: 24 ran 99 us instead of 74 at 512x512x64).
+constexpr int kWarpsFull = 20;
 
 template <int TXP_, int TY_, int S_>
 struct SplitCfg {
@@ -41,6 +44,7 @@ struct SplitCfg {
     static constexpr int NT = (TXP / kStrip) * TY;
     static constexpr int MIN_BLOCKS = kWarpsOneShot * 32 / NT;
     static constexpr int MIN_BLOCKS_BATCHED = kWarpsBatched * 32 / NT;
+    static constexpr int MIN_BLOCKS_FULL = kWarpsFull * 32 / NT;
     static_assert(NT % 32 == 0, "whole warps per CTA");
     using Shape = RingShape<float, TXP, TY, S>;
     static constexpr int BX = Shape::BX;
@@ -147,8 +151,9 @@ __device__ __forceinline__ void st4(float* g, const float* v, int n) {
 // (a k-chunk; it reads one level below and one above). `seq` is the CTA's
 // running load count (CTA-uniform); loads are numbered relative to the
 // lowest level read, lo. Returns false if a bounded wait expired (status
-// set, in-flight loads drained).
-template <class Cfg, bool kVec, bool kLowBits>
+// set, in-flight loads drained). kMeans false (PW_F32): every mean is 0,
+// and the products with the means are left out.
+template <class Cfg, bool kVec, bool kLowBits, bool kMeans>
 __device__ bool split_tile(SplitRing<Cfg, kLowBits>& ring, const CUtensorMap* mu, const CUtensorMap* mv,
                            const CUtensorMap* mw, const FwdArgs& a, int bx, int by, int kb, int ke, long long& seq,
                            int tid) {
@@ -252,53 +257,92 @@ __device__ bool split_tile(SplitRing<Cfg, kLowBits>& ring, const CUtensorMap* mu
             ld4<kVec>(Vu - BX, vus);
             ld4<kVec>(Wu, wu);
         }
-        const float4 t0 = T4[0], t1 = T4[1], t2 = T4[2], t3 = T4[3];
-        const float tcx = T4[6].z, tcy = T4[6].w;
         float r_su[4], r_sv[4], r_sw[4];
+        const float tcx = T4[6].z, tcy = T4[6].w;
+        if constexpr (kMeans) {
+            const float4 t0 = T4[0], t1 = T4[1], t2 = T4[2], t3 = T4[3];
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            const float uw = uj[m], uc = uj[m + 1], ue = uj[m + 2];
-            const float vw = vj[m], vc = vj[m + 1], ve = vj[m + 2];
-            const float wc = wj[m + 1], ww = wj[m], we = wj[m + 2];
-            // su: self term, y cross term, lower vertical flux (table entries 0..6)
-            float p = vs[m] + vs[m + 1], q = vc + ve;
-            float s = tcx * (uw - ue) * (t0.x + uw + uc + ue);
-            s += tcy * (t0.y * (us[m] - un[m + 1]) + t0.z * (p - q) + us[m] * p - un[m + 1] * q);
-            s += t0.w + t1.x * (t1.y * wx_m[m] + t1.z * uo_m[m] + uo_m[m] * wx_m[m]);
-            r_su[m] = s;
-            // sv: mirror (entries 10..15, shared vertical entries 4, 6, 7, 9)
-            p = uw + un[m];
-            q = uc + un[m + 1];
-            s = tcy * (vs[m] - vn[m]) * (t2.z + vs[m] + vc + vn[m]);
-            s += tcx * (t2.w * (vw - ve) + t3.x * (p - q) + vw * p - ve * q);
-            s += t3.y + t1.x * (t3.z * wy_m[m] + t1.z * vo_m[m] + vo_m[m] * wy_m[m]);
-            r_sv[m] = s;
-            const float wx = wc + we, wy = wc + wn[m];
-            float wz = 0.0f;
-            r_sw[m] = 0.0f;
-            if (!top) {
-                const float4 t4 = T4[4], t5 = T4[5], t6 = T4[6];
-                // upper vertical fluxes of su and sv (entries 7, 8, 9, 15)
-                r_su[m] -= t1.w * (t2.x * wx + t2.y * uu[m + 1] + uu[m + 1] * wx);
-                r_sv[m] -= t1.w * (t3.w * wy + t2.y * vu[m] + vu[m] * wy);
-                // sw (entries 16..25)
-                wz = wc + wu[m];
-                p = uw + uu[m];
-                q = uc + uu[m + 1];
-                s = tcx * (t4.x * (p - q) + t4.y * (ww - we) + ww * p - we * q);
-                p = vs[m] + vus[m];
-                q = vc + vu[m];
-                s += tcy * (t4.x * (p - q) + t4.z * (ws[m] - wn[m]) + ws[m] * p - wn[m] * q);
-                s += t4.w + t5.x * (wz_m[m] * (t5.y + wo_m[m]) + t5.z * wo_m[m]);
-                s -= t5.w * (wz * (t6.x + wu[m]) + t6.y * wu[m]);
-                r_sw[m] = s;
+            for (int m = 0; m < 4; ++m) {
+                const float uw = uj[m], uc = uj[m + 1], ue = uj[m + 2];
+                const float vw = vj[m], vc = vj[m + 1], ve = vj[m + 2];
+                const float wc = wj[m + 1], ww = wj[m], we = wj[m + 2];
+                // su: self term, y cross term, lower vertical flux (table entries 0..6)
+                float p = vs[m] + vs[m + 1], q = vc + ve;
+                float s = tcx * (uw - ue) * (t0.x + uw + uc + ue);
+                s += tcy * (t0.y * (us[m] - un[m + 1]) + t0.z * (p - q) + us[m] * p - un[m + 1] * q);
+                s += t0.w + t1.x * (t1.y * wx_m[m] + t1.z * uo_m[m] + uo_m[m] * wx_m[m]);
+                r_su[m] = s;
+                // sv: mirror (entries 10..15, shared vertical entries 4, 6, 7, 9)
+                p = uw + un[m];
+                q = uc + un[m + 1];
+                s = tcy * (vs[m] - vn[m]) * (t2.z + vs[m] + vc + vn[m]);
+                s += tcx * (t2.w * (vw - ve) + t3.x * (p - q) + vw * p - ve * q);
+                s += t3.y + t1.x * (t3.z * wy_m[m] + t1.z * vo_m[m] + vo_m[m] * wy_m[m]);
+                r_sv[m] = s;
+                const float wx = wc + we, wy = wc + wn[m];
+                float wz = 0.0f;
+                r_sw[m] = 0.0f;
+                if (!top) {
+                    const float4 t4 = T4[4], t5 = T4[5], t6 = T4[6];
+                    // upper vertical fluxes of su and sv (entries 7, 8, 9, 15)
+                    r_su[m] -= t1.w * (t2.x * wx + t2.y * uu[m + 1] + uu[m + 1] * wx);
+                    r_sv[m] -= t1.w * (t3.w * wy + t2.y * vu[m] + vu[m] * wy);
+                    // sw (entries 16..25)
+                    wz = wc + wu[m];
+                    p = uw + uu[m];
+                    q = uc + uu[m + 1];
+                    s = tcx * (t4.x * (p - q) + t4.y * (ww - we) + ww * p - we * q);
+                    p = vs[m] + vus[m];
+                    q = vc + vu[m];
+                    s += tcy * (t4.x * (p - q) + t4.z * (ws[m] - wn[m]) + ws[m] * p - wn[m] * q);
+                    s += t4.w + t5.x * (wz_m[m] * (t5.y + wo_m[m]) + t5.z * wo_m[m]);
+                    s -= t5.w * (wz * (t6.x + wu[m]) + t6.y * wu[m]);
+                    r_sw[m] = s;
+                }
+                uo_m[m] = uc;
+                vo_m[m] = vc;
+                wo_m[m] = wc;
+                wx_m[m] = wx;
+                wy_m[m] = wy;
+                wz_m[m] = wz;
             }
-            uo_m[m] = uc;
-            vo_m[m] = vc;
-            wo_m[m] = wc;
-            wx_m[m] = wx;
-            wy_m[m] = wy;
-            wz_m[m] = wz;
+        } else {
+            // PW_F32: of the row only the coefficients are read. Leaving the
+            // products with the means (all 0) out took the 512x512x64 call from
+            // 84 to 74 us (5.4 TB/s, 0.80 of the copy rate) on the same 20
+            // warps per SM, and a batch of 20 domains from 349 to 283 us, where
+            // the persistent kernel now also fits 20 warps instead of 16
+            const float zc1 = T4[1].x, zc2 = T4[1].w, zd1 = T4[5].x, zd2 = T4[5].w;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                const float uw = uj[m], uc = uj[m + 1], ue = uj[m + 2];
+                const float vw = vj[m], vc = vj[m + 1], ve = vj[m + 2];
+                const float wc = wj[m + 1], ww = wj[m], we = wj[m + 2];
+                float s = tcx * (uw - ue) * (uw + uc + ue);
+                s = fmaf(tcy, fmaf(-un[m + 1], vc + ve, us[m] * (vs[m] + vs[m + 1])), s);
+                r_su[m] = fmaf(zc1, uo_m[m] * wx_m[m], s);
+                s = tcy * (vs[m] - vn[m]) * (vs[m] + vc + vn[m]);
+                s = fmaf(tcx, fmaf(-ve, uc + un[m + 1], vw * (uw + un[m])), s);
+                r_sv[m] = fmaf(zc1, vo_m[m] * wy_m[m], s);
+                const float wx = wc + we, wy = wc + wn[m];
+                float wz = 0.0f;
+                r_sw[m] = 0.0f;
+                if (!top) {
+                    r_su[m] = fmaf(-zc2, uu[m + 1] * wx, r_su[m]);
+                    r_sv[m] = fmaf(-zc2, vu[m] * wy, r_sv[m]);
+                    wz = wc + wu[m];
+                    s = tcx * fmaf(-we, uc + uu[m + 1], ww * (uw + uu[m]));
+                    s = fmaf(tcy, fmaf(-wn[m], vc + vu[m], ws[m] * (vs[m] + vus[m])), s);
+                    s = fmaf(zd1, wz_m[m] * wo_m[m], s);
+                    r_sw[m] = fmaf(-zd2, wz * wu[m], s);
+                }
+                uo_m[m] = uc;
+                vo_m[m] = vc;
+                wo_m[m] = wc;
+                wx_m[m] = wx;
+                wy_m[m] = wy;
+                wz_m[m] = wz;
+            }
         }
         if (nval > 0) {
             st4<kVec>(su + g, r_su, nval);
@@ -323,11 +367,10 @@ __device__ bool split_tile(SplitRing<Cfg, kLowBits>& ring, const CUtensorMap* mu
     return true;
 }
 
-template <class Cfg, bool kVec>
-__global__ void __launch_bounds__(Cfg::NT, Cfg::MIN_BLOCKS) fwd_split_kernel(const __grid_constant__ CUtensorMap mu,
-                                                            const __grid_constant__ CUtensorMap mv,
-                                                            const __grid_constant__ CUtensorMap mw,
-                                                            const FwdArgs a, const ItemSched sched) {
+template <class Cfg, bool kVec, bool kFull>
+__global__ void __launch_bounds__(Cfg::NT, kFull ? Cfg::MIN_BLOCKS_FULL : Cfg::MIN_BLOCKS)
+    fwd_split_kernel(const __grid_constant__ CUtensorMap mu, const __grid_constant__ CUtensorMap mv,
+                     const __grid_constant__ CUtensorMap mw, const FwdArgs a, const ItemSched sched) {
     extern __shared__ unsigned char smem_raw[];
     SplitRing<Cfg, true> ring;
     ring.setup(smem_raw);
@@ -342,13 +385,13 @@ __global__ void __launch_bounds__(Cfg::NT, Cfg::MIN_BLOCKS) fwd_split_kernel(con
     long long seq = 0;
     int bx, by, k0, k1;
     sched_item(sched, a.kend - a.kbeg, blockIdx.x, &bx, &by, &k0, &k1);
-    (void)split_tile<Cfg, kVec, true>(ring, &mu, &mv, &mw, a, bx, by, a.kbeg + k0, a.kbeg + k1, seq, tid);
+    (void)split_tile<Cfg, kVec, true, !kFull>(ring, &mu, &mv, &mw, a, bx, by, a.kbeg + k0, a.kbeg + k1, seq, tid);
 }
 
 // Persistent form: the CTA takes work items (one k-chunk of one tile of one
 // domain) from the plan's counter until none are left; at most n_items
 // iterations. Items are ordered by the plan builder (taller columns first).
-template <class Cfg, bool kVec>
+template <class Cfg, bool kVec, bool kFull>
 __device__ __forceinline__ void run_items(BatchPlan* plan, SplitRing<Cfg>& ring, int tid) {
     const long long n_items = plan->n_items;
     long long seq = 0;
@@ -368,13 +411,15 @@ __device__ __forceinline__ void run_items(BatchPlan* plan, SplitRing<Cfg>& ring,
         const int ch = (int)(t / tiles), tt = (int)(t % tiles);
         const int kb = (int)((long long)args.nz * ch / kchunks);
         const int ke = (int)((long long)args.nz * (ch + 1) / kchunks);
-        if (!split_tile<Cfg, kVec, false>(ring, &d.mu, &d.mv, &d.mw, args, tt % tiles_x, tt / tiles_x, kb, ke, seq, tid))
+        if (!split_tile<Cfg, kVec, false, !kFull>(ring, &d.mu, &d.mv, &d.mw, args, tt % tiles_x, tt / tiles_x, kb, ke,
+                                                  seq, tid))
             break;
     }
 }
 
-template <class Cfg>
-__global__ void __launch_bounds__(Cfg::NT, Cfg::MIN_BLOCKS_BATCHED) fwd_split_batched(BatchPlan* plan, int variant) {
+template <class Cfg, bool kFull>
+__global__ void __launch_bounds__(Cfg::NT, kFull ? Cfg::MIN_BLOCKS_FULL : Cfg::MIN_BLOCKS_BATCHED)
+    fwd_split_batched(BatchPlan* plan, int variant) {
     extern __shared__ unsigned char smem_raw[];
     SplitRing<Cfg> ring;
     ring.setup(smem_raw);
@@ -386,8 +431,8 @@ __global__ void __launch_bounds__(Cfg::NT, Cfg::MIN_BLOCKS_BATCHED) fwd_split_ba
     if (tid == 0) ring.init_barriers();
     __syncthreads();
     // one whole item loop per path, chosen once, so each gets the registers to itself
-    if (plan->all_vec) run_items<Cfg, true>(plan, ring, tid);
-    else run_items<Cfg, false>(plan, ring, tid);
+    if (plan->all_vec) run_items<Cfg, true, kFull>(plan, ring, tid);
+    else run_items<Cfg, false, kFull>(plan, ring, tid);
 }
 
 // Tile-shape / pipeline-depth variants (the autotuner's search space).
@@ -405,10 +450,10 @@ TileShape shape_of() {
     return TileShape{Cfg::TXP, Cfg::TY, Cfg::BX, Cfg::Shape::BY, Cfg::SMEM_BYTES, Cfg::NT};
 }
 
-template <class Cfg>
+template <class Cfg, bool kFull>
 cudaError_t launch_one(const CUtensorMap& mu, const CUtensorMap& mv, const CUtensorMap& mw, const FwdArgs& a,
                        cudaStream_t st) {
-    auto kern = a.vec ? fwd_split_kernel<Cfg, true> : fwd_split_kernel<Cfg, false>;
+    auto kern = a.vec ? fwd_split_kernel<Cfg, true, kFull> : fwd_split_kernel<Cfg, false, kFull>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     ItemSched sched;
@@ -419,9 +464,9 @@ cudaError_t launch_one(const CUtensorMap& mu, const CUtensorMap& mv, const CUten
     return cudaGetLastError();
 }
 
-template <class Cfg>
+template <class Cfg, bool kFull>
 cudaError_t launch_batched_cfg(int v, BatchPlan* plan, long long n_items, cudaStream_t st) {
-    auto kern = fwd_split_batched<Cfg>;
+    auto kern = fwd_split_batched<Cfg, kFull>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
     if (e != cudaSuccess) return e;
     long long grid = 0;
@@ -429,6 +474,20 @@ cudaError_t launch_batched_cfg(int v, BatchPlan* plan, long long n_items, cudaSt
     if (grid < 1) return cudaSuccess;
     kern<<<(unsigned)grid, Cfg::NT, Cfg::SMEM_BYTES, st>>>(plan, v);
     return cudaGetLastError();
+}
+
+template <bool kFull>
+cudaError_t launch_batched_variant(int v, BatchPlan* plan, long long n_items, cudaStream_t st) {
+    switch (v) {
+        case 1: return launch_batched_cfg<V1, kFull>(1, plan, n_items, st);
+        case 2: return launch_batched_cfg<V2, kFull>(2, plan, n_items, st);
+        case 3: return launch_batched_cfg<V3, kFull>(3, plan, n_items, st);
+        case 4: return launch_batched_cfg<V4, kFull>(4, plan, n_items, st);
+        case 5: return launch_batched_cfg<V5, kFull>(5, plan, n_items, st);
+        case 6: return launch_batched_cfg<V6, kFull>(6, plan, n_items, st);
+        case 7: return launch_batched_cfg<V7, kFull>(7, plan, n_items, st);
+        default: return launch_batched_cfg<V0, kFull>(0, plan, n_items, st);
+    }
 }
 
 }  // namespace
@@ -454,36 +513,13 @@ TileShape fwd_split_shape_variant(int v) {
 
 TileShape fwd_split_shape() { return fwd_split_shape_variant(0); }
 
-cudaError_t launch_fwd_split_variant(int v, const CUtensorMap& mu, const CUtensorMap& mv, const CUtensorMap& mw,
-                                     const FwdArgs& a, cudaStream_t st) {
-    switch (v) {
-        case 1: return launch_one<V1>(mu, mv, mw, a, st);
-        case 2: return launch_one<V2>(mu, mv, mw, a, st);
-        case 3: return launch_one<V3>(mu, mv, mw, a, st);
-        case 4: return launch_one<V4>(mu, mv, mw, a, st);
-        case 5: return launch_one<V5>(mu, mv, mw, a, st);
-        case 6: return launch_one<V6>(mu, mv, mw, a, st);
-        case 7: return launch_one<V7>(mu, mv, mw, a, st);
-        default: return launch_one<V0>(mu, mv, mw, a, st);
-    }
-}
-
-cudaError_t launch_fwd_split(const CUtensorMap& mu, const CUtensorMap& mv, const CUtensorMap& mw,
+cudaError_t launch_fwd_split(bool full, const CUtensorMap& mu, const CUtensorMap& mv, const CUtensorMap& mw,
                              const FwdArgs& a, cudaStream_t st) {
-    return launch_fwd_split_variant(0, mu, mv, mw, a, st);
+    return full ? launch_one<V0, true>(mu, mv, mw, a, st) : launch_one<V0, false>(mu, mv, mw, a, st);
 }
 
-cudaError_t launch_split_batched(int v, BatchPlan* plan, long long n_items, cudaStream_t st) {
-    switch (v) {
-        case 1: return launch_batched_cfg<V1>(1, plan, n_items, st);
-        case 2: return launch_batched_cfg<V2>(2, plan, n_items, st);
-        case 3: return launch_batched_cfg<V3>(3, plan, n_items, st);
-        case 4: return launch_batched_cfg<V4>(4, plan, n_items, st);
-        case 5: return launch_batched_cfg<V5>(5, plan, n_items, st);
-        case 6: return launch_batched_cfg<V6>(6, plan, n_items, st);
-        case 7: return launch_batched_cfg<V7>(7, plan, n_items, st);
-        default: return launch_batched_cfg<V0>(0, plan, n_items, st);
-    }
+cudaError_t launch_split_batched(bool full, int v, BatchPlan* plan, long long n_items, cudaStream_t st) {
+    return full ? launch_batched_variant<true>(v, plan, n_items, st) : launch_batched_variant<false>(v, plan, n_items, st);
 }
 
 }  // namespace pw

@@ -295,6 +295,13 @@ def fill_periodic_halo(f, nx, ny, stream=None):
     return f
 
 
+def _arithmetic(mode, split_table):
+    """The library dtype of a mode. PW_F32 reads only the coefficients of its
+    table, so a table of the caller's own, which may hold means, goes through
+    the mean + perturbation arithmetic."""
+    return PW_F32_SPLIT if mode == "f32" and split_table is not None else MODES[mode]
+
+
 def advect(u, v, w, coeffs: Coefficients, nx, ny, mode="paired", split_table=None, out=None, stream=None):
     """Source terms (su, sv, sw) of u, v, w.
 
@@ -303,7 +310,7 @@ def advect(u, v, w, coeffs: Coefficients, nx, ny, mode="paired", split_table=Non
     device table from :func:`make_split_table`) or "f32" (float full fields).
     """
     lib = load_library()
-    dt = MODES[mode]
+    dt = _arithmetic(mode, split_table)
     if mode == "f32" and split_table is None:
         split_table = coeffs.zero_mean_table(u.device)
     d = dims_of(u, nx, ny)
@@ -384,7 +391,7 @@ def advect_host(u_h, v_h, w_h, coeffs: Coefficients, nx, ny, mode="paired", out_
     must be complete in host memory when the call is made."""
     import torch
     lib = load_library()
-    dt = MODES[mode]
+    dt = _arithmetic(mode, split_table)
     nz = u_h.shape[0]
     d = dims_of(u_h, nx, ny)
     own = pipeline is None
@@ -589,7 +596,8 @@ class Batch:
         import torch
         lib = load_library()
         self.mode, self.variant = mode, int(variant)
-        self.dt = MODES[mode]
+        self.dt = max((_arithmetic(mode, d.get("split_table")) for d in domains), key=lambda a: a == PW_F32_SPLIT,
+                      default=MODES[mode])
         self.domains = []
         cs = (Domain * len(domains))()
         for n, d in enumerate(domains):
