@@ -47,7 +47,7 @@ extern "C" {
 #define PW_ETIMEOUT (-6)      /* a kernel's bounded wait expired (see pw_device_status) */
 
 typedef enum {
-    PW_F64 = 0,        /* double in, double out, native FP64 arithmetic */
+    PW_F64 = 0,        /* double in, double out, FP64 accuracy at least */
     PW_F32_SPLIT = 1,  /* float perturbations about per-level means, FP32 arithmetic */
     PW_F64_PAIRED = 2, /* double in, double out, paired-FP32 (double-float) arithmetic */
     PW_F32 = 3         /* float in, float out, FP32 arithmetic on the full fields */
@@ -118,9 +118,12 @@ int pw_fill_periodic_halo(pw_dtype dtype, void *field, const pw_dims *dims, void
  *   be NULL. Error scales at a point: A = sum over the face terms c*q*(a+b)
  *   of |c||q||a+b| (the absolute values of the products the formula adds);
  *   M = the same with |a|+|b| in place of |a+b| (M >= A).
- *   PW_F64 computes in FP64, each operation rounded once (u and v are scaled
- *   by tcx and tcy once per cell, then every face sum is formed once and
- *   shared); its error is a few units of 2^-53 of M, within 1e-13 of A.
+ *   PW_F64 (forward): sums of products in 87-bit fixed point, split from the
+ *   doubles without error, each output rounded to double once and multiplied
+ *   by the larger of tcx and tcy; values that the fixed point cannot hold
+ *   beside their neighbours, infinities and NaN make the outputs that read
+ *   them, or their neighbours, native FP64 evaluations term by term. Its error
+ *   is a few units of 2^-53 of M, within 1e-13 of A.
  *   PW_F64_PAIRED carries every value as an unevaluated sum of two floats
  *   (about 48 significant bits); each double is split into a pair before
  *   a + b is formed, so its error is bounded by M: within 1e-13 of M at
@@ -281,7 +284,7 @@ size_t pw_batch_plan_bytes(int n);
  * 1 = 64x4; 2 = 32x8; 3 = 64x8; 4 = 32x16; 5 = 128x2 (all 4 levels);
  * 6 = 64x4, 3 levels; 7 = 64x4, 6 levels.
  * PW_F64_PAIRED: 0 = 32x8, 2 levels; 1 = 32x4; 2 = 32x16 (2 levels);
- * 3 = 32x8, 3 levels. PW_F64: 0 = 32x16, 1 = 32x8 (4-level rings). */
+ * 3 = 32x8, 3 levels. PW_F64: 0 and 1 are the same kernel (32x16). */
 int pw_variant_count(pw_dtype dtype);
 
 /*

@@ -302,11 +302,15 @@ static int advect_levels(pw_dtype dtype, const void* u, const void* v, const voi
     a.sz = dims->sz;
     a.tcx = c->tcx;
     a.tcy = c->tcy;
+    pw::set_reference(a);
     a.tzc1 = c->tzc1;
     a.tzc2 = c->tzc2;
     a.tzd1 = c->tzd1;
     a.tzd2 = c->tzd2;
     a.split = static_cast<const float*>(split);
+    a.u = u;
+    a.v = v;
+    a.w = w;
     a.su = su;
     a.sv = sv;
     a.sw = sw;
@@ -633,11 +637,15 @@ extern "C" int pw_make_batch_plan(pw_dtype dtype, int n, const pw_domain* doms, 
             if (((uintptr_t)ptrs[k] + es) % 16 != 0) a.vec = 0;
         a.tcx = dm.coeffs.tcx;
         a.tcy = dm.coeffs.tcy;
+        pw::set_reference(a);
         a.tzc1 = dm.coeffs.tzc1;
         a.tzc2 = dm.coeffs.tzc2;
         a.tzd1 = dm.coeffs.tzd1;
         a.tzd2 = dm.coeffs.tzd2;
         a.split = static_cast<const float*>(dm.split);
+        a.u = dm.u;
+        a.v = dm.v;
+        a.w = dm.w;
         a.su = dm.su;
         a.sv = dm.sv;
         a.sw = dm.sw;

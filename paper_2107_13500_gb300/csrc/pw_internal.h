@@ -5,6 +5,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <cmath>
 #include <cstddef>
 #include <map>
 #include <mutex>
@@ -19,10 +20,26 @@ struct FwdArgs {
     int xoff;                  // elements from the descriptors' 16-byte base to i = 0
     int vec;                   // 1: every field's interior i = 1 starts on 16 bytes
     double tcx, tcy;
+    double tref, tinv;         // PW_F64: the larger of tcx and tcy in magnitude, and 1 / tref
+    int same_t, limbs;         // tcx = tcy; tcx, tcy and tref suit the limb arithmetic
     const double *tzc1, *tzc2, *tzd1, *tzd2;
     const float* split;        // PW_F32_SPLIT table, else nullptr
+    const void *u, *v, *w;     // the fields, for points that read them with plain loads
     void *su, *sv, *sw;
 };
+
+// tref, tinv, same_t and limbs from tcx and tcy: 1 / tref must be normal, and
+// where tcx and tcy differ, each over tref 0 or at least 2^-30.
+inline void set_reference(FwdArgs& a) {
+    a.same_t = a.tcx == a.tcy ? 1 : 0;
+    a.tref = std::fabs(a.tcx) >= std::fabs(a.tcy) ? a.tcx : a.tcy;
+    const double m = std::fabs(a.tref);
+    a.limbs = m >= 0x1p-300 && m <= 0x1p300 ? 1 : 0;  // (false for NaN)
+    a.tinv = a.limbs ? 1.0 / a.tref : 1.0;
+    if (!a.same_t)
+        for (double t : {a.tcx, a.tcy})
+            if (!(t == 0.0 || std::fabs(t * a.tinv) >= 0x1p-30)) a.limbs = 0;
+}
 
 // Tile shape of each forward kernel (the host builds TMA boxes to match).
 struct TileShape {
