@@ -307,7 +307,9 @@ __device__ bool split_tile(SplitRing<Cfg, kLowBits>& ring, const CUtensorMap* mu
                 wz_m[m] = wz;
             }
         } else {
-            // PW_F32: of the row only the coefficients are read. Leaving the
+            // PW_F32: of the row only the coefficients are read (every operation
+            // rounds as with means of 0 in the form above, so the results are
+            // the same bits). Leaving the
             // products with the means (all 0) out took the 512x512x64 call from
             // 84 to 74 us (5.4 TB/s, 0.80 of the copy rate) on the same 20
             // warps per SM, and a batch of 20 domains from 349 to 283 us, where
@@ -318,12 +320,13 @@ __device__ bool split_tile(SplitRing<Cfg, kLowBits>& ring, const CUtensorMap* mu
                 const float uw = uj[m], uc = uj[m + 1], ue = uj[m + 2];
                 const float vw = vj[m], vc = vj[m + 1], ve = vj[m + 2];
                 const float wc = wj[m + 1], ww = wj[m], we = wj[m + 2];
-                float s = tcx * (uw - ue) * (uw + uc + ue);
-                s = fmaf(tcy, fmaf(-un[m + 1], vc + ve, us[m] * (vs[m] + vs[m + 1])), s);
-                r_su[m] = fmaf(zc1, uo_m[m] * wx_m[m], s);
-                s = tcy * (vs[m] - vn[m]) * (vs[m] + vc + vn[m]);
-                s = fmaf(tcx, fmaf(-ve, uc + un[m + 1], vw * (uw + un[m])), s);
-                r_sv[m] = fmaf(zc1, vo_m[m] * wy_m[m], s);
+                float x = __fmul_rn(tcx, uw - ue), y = fmaf(-un[m + 1], vc + ve, us[m] * (vs[m] + vs[m + 1]));
+                float s = fmaf(x, uw + uc + ue, __fmul_rn(tcy, y));
+                r_su[m] = __fadd_rn(s, __fmul_rn(zc1, uo_m[m] * wx_m[m]));
+                y = __fmul_rn(tcy, vs[m] - vn[m]);
+                x = fmaf(-ve, uc + un[m + 1], vw * (uw + un[m]));
+                s = fmaf(y, vs[m] + vc + vn[m], __fmul_rn(tcx, x));
+                r_sv[m] = __fadd_rn(s, __fmul_rn(zc1, vo_m[m] * wy_m[m]));
                 const float wx = wc + we, wy = wc + wn[m];
                 float wz = 0.0f;
                 r_sw[m] = 0.0f;
@@ -331,9 +334,9 @@ __device__ bool split_tile(SplitRing<Cfg, kLowBits>& ring, const CUtensorMap* mu
                     r_su[m] = fmaf(-zc2, uu[m + 1] * wx, r_su[m]);
                     r_sv[m] = fmaf(-zc2, vu[m] * wy, r_sv[m]);
                     wz = wc + wu[m];
-                    s = tcx * fmaf(-we, uc + uu[m + 1], ww * (uw + uu[m]));
-                    s = fmaf(tcy, fmaf(-wn[m], vc + vu[m], ws[m] * (vs[m] + vus[m])), s);
-                    s = fmaf(zd1, wz_m[m] * wo_m[m], s);
+                    x = fmaf(-we, uc + uu[m + 1], ww * (uw + uu[m]));
+                    y = fmaf(-wn[m], vc + vu[m], ws[m] * (vs[m] + vus[m]));
+                    s = __fadd_rn(fmaf(tcx, x, __fmul_rn(tcy, y)), __fmul_rn(zd1, wz_m[m] * wo_m[m]));
                     r_sw[m] = fmaf(-zd2, wz * wu[m], s);
                 }
                 uo_m[m] = uc;
