@@ -66,13 +66,16 @@ class Domain(ctypes.Structure):
 
 _lock = threading.Lock()
 _lib = None
+_raw_stream = None  # torch's current cudaStream_t by device index, where this torch has it
 _dp = ctypes.POINTER(ctypes.c_double)
 _fp = ctypes.POINTER(ctypes.c_float)
 
 
 def load_library(path: str | None = None):
     """Load libpw.so (built by ``build.build()``); raise if it is missing."""
-    global _lib
+    global _lib, _raw_stream
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -126,6 +129,12 @@ def load_library(path: str | None = None):
         lib.pw_euler_periodic_adjoint.argtypes = [ctypes.c_int] + [vp] * 3 + [ctypes.c_double, ctypes.POINTER(Dims),
                                                                               ctypes.c_int] + [vp] * 7
         lib.pw_euler_periodic_adjoint.restype = ctypes.c_int
+        try:
+            import torch
+            if hasattr(torch._C, "_cuda_getDevice"):
+                _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        except ImportError:
+            pass
         _lib = lib
         return lib
 
@@ -215,9 +224,17 @@ def dims_of(t, nx: int, ny: int) -> Dims:
 
 
 def _stream_handle(stream=None):
+    return ctypes.c_void_p(_stream_ptr(stream))
+
+
+def _stream_ptr(stream=None):
+    """The cudaStream_t of a torch stream (default: the current stream) as an int."""
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch._C._cuda_getDevice())  # without building a Stream object
+    return torch.cuda.current_stream().cuda_stream
 
 
 # ---------------------------------------------------------------- coefficients
@@ -249,8 +266,8 @@ class Coefficients:
     def c_struct(self) -> Coeffs:
         if self.dev is None:
             self.to_device()
-        d = self.dev
-        return Coeffs(self.tcx, self.tcy, d[0].data_ptr(), d[1].data_ptr(), d[2].data_ptr(), d[3].data_ptr())
+        base, row = self.dev.data_ptr(), 8 * self.dev.stride(0)
+        return Coeffs(self.tcx, self.tcy, base, base + row, base + 2 * row, base + 3 * row)
 
     def as_dict(self):
         return dict(tcx=self.tcx, tcy=self.tcy, tzc1=self.tz4[0], tzc2=self.tz4[1], tzd1=self.tz4[2],
@@ -291,7 +308,7 @@ def fill_periodic_halo(f, nx, ny, stream=None):
     dt = PW_F32_SPLIT if f.dtype == torch.float32 else PW_F64
     d = dims_of(f, nx, ny)
     _check(load_library().pw_fill_periodic_halo(dt, ctypes.c_void_p(f.data_ptr()), ctypes.byref(d),
-                                                _stream_handle(stream)))
+                                                _stream_ptr(stream)))
     return f
 
 
@@ -314,21 +331,20 @@ def advect(u, v, w, coeffs: Coefficients, nx, ny, mode="paired", split_table=Non
     if mode == "f32" and split_table is None:
         split_table = coeffs.zero_mean_table(u.device)
     d = dims_of(u, nx, ny)
+    layout = (u.shape, u.stride(), u.dtype)
     for t in (v, w):
-        if t.shape != u.shape or t.stride() != u.stride() or t.dtype != u.dtype:
+        if (t.shape, t.stride(), t.dtype) != layout:
             raise ValueError("u, v, w must share shape, strides and dtype")
     if out is None:
         out = tuple(field_like(u) for _ in range(3))
     su, sv, sw = out
     for t in out:
-        if t.shape != u.shape or t.stride() != u.stride() or t.dtype != u.dtype:
+        if (t.shape, t.stride(), t.dtype) != layout:
             raise ValueError("outputs must match the inputs' layout")
     c = coeffs.c_struct()
-    sp = None if split_table is None else ctypes.c_void_p(split_table.data_ptr())
-    _check(lib.pw_advect(dt, ctypes.c_void_p(u.data_ptr()), ctypes.c_void_p(v.data_ptr()),
-                         ctypes.c_void_p(w.data_ptr()), ctypes.byref(c), ctypes.byref(d), sp,
-                         ctypes.c_void_p(su.data_ptr()), ctypes.c_void_p(sv.data_ptr()),
-                         ctypes.c_void_p(sw.data_ptr()), _stream_handle(stream)))
+    _check(lib.pw_advect(dt, u.data_ptr(), v.data_ptr(), w.data_ptr(), ctypes.byref(c), ctypes.byref(d),
+                         None if split_table is None else split_table.data_ptr(), su.data_ptr(), sv.data_ptr(),
+                         sw.data_ptr(), _stream_ptr(stream)))
     return su, sv, sw
 
 
@@ -446,7 +462,7 @@ def split_field(f, nx, ny, out=None, mean=None, stream=None):
     dp = dims_of(fp, nx, ny)
     m = mean if mean is not None else torch.empty(f.shape[0], dtype=torch.float64, device=f.device)
     _check(lib.pw_split_field(ctypes.c_void_p(f.data_ptr()), ctypes.byref(df), ctypes.c_void_p(fp.data_ptr()),
-                              ctypes.byref(dp), ctypes.c_void_p(m.data_ptr()), _stream_handle(stream)))
+                              ctypes.byref(dp), ctypes.c_void_p(m.data_ptr()), _stream_ptr(stream)))
     return fp, m
 
 
@@ -454,13 +470,13 @@ def selftest_bounded_wait(limit_us=20000, stream=None) -> int:
     """Run the bounded-wait self-test; returns the status it left
     (PW_ETIMEOUT when waits are bounded)."""
     st = ctypes.c_int(0)
-    _check(load_library().pw_selftest_bounded_wait(int(limit_us), ctypes.byref(st), _stream_handle(stream)))
+    _check(load_library().pw_selftest_bounded_wait(int(limit_us), ctypes.byref(st), _stream_ptr(stream)))
     return st.value
 
 
 def device_status(stream=None) -> int:
     st = ctypes.c_int(0)
-    _check(load_library().pw_device_status(ctypes.byref(st), _stream_handle(stream)))
+    _check(load_library().pw_device_status(ctypes.byref(st), _stream_ptr(stream)))
     return st.value
 
 
@@ -474,17 +490,17 @@ def advect_adjoint(u, v, w, coeffs: Coefficients, nx, ny, gsu, gsv, gsw, mode="f
     dt = {"f64": PW_F64, "paired": PW_F64_PAIRED, "f32": PW_F32}[mode]
     d = dims_of(u, nx, ny)
     ins = (u, v, w, gsu, gsv, gsw)
+    layout = (u.shape, u.stride(), u.dtype)
     for t in ins[1:]:
-        if t.shape != u.shape or t.stride() != u.stride() or t.dtype != u.dtype:
+        if (t.shape, t.stride(), t.dtype) != layout:
             raise ValueError("u, v, w and the cotangents must share shape, strides and dtype")
     if out is None:
         out = tuple(field_like(u) for _ in range(3))
     gu, gv, gw = out
     c = coeffs.c_struct()
-    vp = ctypes.c_void_p
-    _check(lib.pw_advect_adjoint(dt, *(vp(t.data_ptr()) for t in ins[:3]), ctypes.byref(c), ctypes.byref(d),
-                                 *(vp(t.data_ptr()) for t in ins[3:]), vp(gu.data_ptr()), vp(gv.data_ptr()),
-                                 vp(gw.data_ptr()), 1 if accumulate else 0, _stream_handle(stream)))
+    p = [t.data_ptr() for t in ins]
+    _check(lib.pw_advect_adjoint(dt, *p[:3], ctypes.byref(c), ctypes.byref(d), *p[3:], gu.data_ptr(), gv.data_ptr(),
+                                 gw.data_ptr(), 1 if accumulate else 0, _stream_ptr(stream)))
     return gu, gv, gw
 
 
@@ -526,7 +542,7 @@ def energy_budget(u, v, w, su, sv, sw, nx, ny, wu, ww, stream=None):
     _check(lib.pw_energy_budget(vp(u.data_ptr()), vp(v.data_ptr()), vp(w.data_ptr()), u.element_size(),
                                 ctypes.byref(dw), vp(su.data_ptr()), vp(sv.data_ptr()), vp(sw.data_ptr()),
                                 su.element_size(), ctypes.byref(ds), vp(wu.data_ptr()), vp(ww.data_ptr()),
-                                vp(level.data_ptr()), vp(totals.data_ptr()), _stream_handle(stream)))
+                                vp(level.data_ptr()), vp(totals.data_ptr()), _stream_ptr(stream)))
     return totals, level
 
 
@@ -537,7 +553,7 @@ def fold_periodic_halo(g, nx, ny, stream=None):
     dt = PW_F32 if g.dtype == torch.float32 else PW_F64
     d = dims_of(g, nx, ny)
     _check(load_library().pw_fold_periodic_halo(dt, ctypes.c_void_p(g.data_ptr()), ctypes.byref(d),
-                                                _stream_handle(stream)))
+                                                _stream_ptr(stream)))
     return g
 
 
@@ -560,7 +576,7 @@ def euler_periodic(fields, tendencies, dt, nx, ny, stream=None):
     vp = ctypes.c_void_p
     _check(load_library().pw_euler_periodic(dtype, *(vp(t.data_ptr()) for t in tuple(fields) + tuple(tendencies)),
                                             float(dt), ctypes.byref(d), fields[0].shape[2],
-                                            *(vp(t.data_ptr()) for t in out), _stream_handle(stream)))
+                                            *(vp(t.data_ptr()) for t in out), _stream_ptr(stream)))
     return out
 
 
@@ -572,7 +588,7 @@ def euler_periodic_adjoint(grads, dt, nx, ny, like, stream=None):
     vp = ctypes.c_void_p
     _check(load_library().pw_euler_periodic_adjoint(dtype, *(vp(t.data_ptr()) for t in grads), float(dt),
                                                     ctypes.byref(d), like.shape[2],
-                                                    *(vp(t.data_ptr()) for t in gf + gs), _stream_handle(stream)))
+                                                    *(vp(t.data_ptr()) for t in gf + gs), _stream_ptr(stream)))
     return gf, gs
 
 
@@ -627,7 +643,7 @@ class Batch:
 
     def run(self, stream=None):
         _check(load_library().pw_advect_batched(self.dt, self.variant, ctypes.c_void_p(self.plan_dev.data_ptr()),
-                                                self.n_items, _stream_handle(stream)))
+                                                self.n_items, _stream_ptr(stream)))
 
     def outputs(self):
         return [(d["su"], d["sv"], d["sw"]) for d in self.domains]
