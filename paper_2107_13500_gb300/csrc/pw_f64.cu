@@ -49,11 +49,14 @@
 // FP64 pipe 16 %, DRAM 19 %. Neither more warps (96 registers, 20 warps), nor
 // shorter chains (separate sums of each limb product), nor the multiply-add as
 // a product and an addition (half rate, one instruction more) moved it by more
-// than 3 %. 512x512x64 without density: 1043 -> 560 us (30 GPt/s); with density
-// 1138 -> 591 us; 1000x250x37 with density, tcx != tcy, unaligned: 659 -> 384 us;
-// 128x128x64: 82 -> 53 us; a batch of 20 domains: 3877 -> 2027 us. Winds of
-// 1e3 or 1e-3 times that size take 575 and 618 us. A column of FP64 steps costs
-// about 1650 us at 512x512x64, more than before.
+// than 3 %. A tile's first three levels are copied at once, two of them into limb
+// slots not yet in use, before the scan of the coefficients (one after another
+// through the stage: 562 us at 512x512x64, 157 at 256x256x64 where it is now 150).
+// 512x512x64 without density: 1043 -> 543 us (31 GPt/s); with density 1138 -> 571
+// us; 1000x250x37 with density, tcx != tcy, unaligned: 658 -> 370 us; 128x128x64:
+// 82 -> 45 us; a batch of 20 domains: 3879 -> 2078 us. Winds of 1e3 or 1e-3 times
+// that size take 557 and 623 us. A column of FP64 steps costs about 1650 us at
+// 512x512x64, more than before.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -90,8 +93,14 @@ struct F64Cfg {
     static constexpr int COEF_OFFSET = LIMB_OFFSET + SLOTS * SLOT * 16;
     static constexpr int ITEM_OFFSET = COEF_OFFSET + 4 * 4 * 16;
     static constexpr int SMEM_BYTES = ITEM_OFFSET + 32 + 128;
-    static_assert(S * 8 <= 64, "ring barriers must fit before the limbs");
+    static_assert((S + 2) * 8 <= 64, "ring and start barriers must fit before the limbs");
     static_assert(MINB * (SMEM_BYTES + 1024) <= 228 * 1024, "CTAs per SM");
+    // While a tile starts, its first two levels arrive in limb slots 1 and 2 (not
+    // yet in use), the third in the stage, so that the three copies overlap.
+    static constexpr int RAW1 = round_up(LIMB_OFFSET + SLOT * 16, 128), RAW2 = round_up(LIMB_OFFSET + 2 * SLOT * 16, 128);
+    static_assert(S == 1 && RAW1 + Shape::STAGE_BYTES <= LIMB_OFFSET + 2 * SLOT * 16 &&
+                      RAW2 + Shape::STAGE_BYTES <= LIMB_OFFSET + 3 * SLOT * 16,
+                  "a level's boxes fit a limb slot");
     static_assert(SLOT < 65536 && 3 * Shape::BOX_STRIDE / 8 < 65536, "offsets of a plan fit 16 bits");
 };
 
@@ -114,6 +123,41 @@ struct F64K {
         sm.item = reinterpret_cast<long long*>(ring.base + C::ITEM_OFFSET);
         sm.range = reinterpret_cast<int*>(ring.base + C::ITEM_OFFSET + 8);
         sm.big = reinterpret_cast<unsigned*>(ring.base + C::ITEM_OFFSET + 16);
+    }
+
+    // The ring's barrier, and one for each of a tile's first two levels.
+    static __device__ __forceinline__ void init_barriers(Ring<Shape>& ring) {
+        mbar_init(&ring.full[1], 1);
+        mbar_init(&ring.full[2], 1);
+        ring.init_barriers();
+    }
+
+    // Where a CTA stands: loads by level (tags of the limb slots), loads through
+    // the ring, and the phases of the two start barriers.
+    struct Counts {
+        long long levels = 0, ring = 0;
+        unsigned phase1 = 0, phase2 = 0;
+    };
+
+    // Levels read by a chunk kb..ke-1: one below, one above.
+    static __device__ __forceinline__ int lowest(int kb) { return kb > 0 ? kb - 1 : 0; }
+    static __device__ __forceinline__ int highest(const FwdArgs& a, int ke) { return ke < a.nz ? ke : a.nz - 1; }
+
+    // Issue a tile's first three levels (one thread).
+    static __device__ __forceinline__ void start_tile(Ring<Shape>& ring, const CUtensorMap* mu, const CUtensorMap* mv,
+                                                      const CUtensorMap* mw, const FwdArgs& a, int bx, int by, int kb,
+                                                      int ke, const Counts& n) {
+        const int x0 = bx * C::TX, y0 = by * C::TY, lo = lowest(kb), nl = highest(a, ke) - lo + 1;
+        fence_proxy_async_smem();
+        for (int r = 0; r < 2 && r < nl; ++r) {
+            uint64_t* bar = &ring.full[1 + r];
+            unsigned char* dst = ring.base + (r == 0 ? C::RAW1 : C::RAW2);
+            mbar_arrive_expect_tx(bar, 3 * Shape::BOX_BYTES);
+            tma_load_3d(dst, mu, bar, x0, y0, lo + r);
+            tma_load_3d(dst + Shape::BOX_STRIDE, mv, bar, x0, y0, lo + r);
+            tma_load_3d(dst + 2 * Shape::BOX_STRIDE, mw, bar, x0, y0, lo + r);
+        }
+        if (nl > 2) ring.issue((long long)(unsigned)n.ring, lo + 2, mu, mv, mw, x0, y0);
     }
 
     // What the coefficient arrays of a domain allow: equal lower and upper
@@ -208,13 +252,14 @@ struct F64K {
         return __ldg(arr + lev);
     }
 
-    // Split load `seq` (level lev) into limb slot `slot` at scale z; false where
-    // a value is outside its window. Tells the CTA where one lies in the scale's
+    // Split the staged boxes of level lev into limb slot `slot` at scale z (tag:
+    // the level's number in the CTA's loads); false where a value is outside its
+    // window. Tells the CTA where one lies in the scale's
     // own binades (the top kLimbStep of the window).
-    static __device__ __forceinline__ bool split_level(const Ring<Shape>& ring, const Smem& sm, long long seq, int lev,
+    static __device__ __forceinline__ bool split_level(const unsigned char* stage, const Smem& sm, unsigned tag, int lev,
                                                        int slot, int z, const FwdArgs& a, int delta, int tid,
                                                        const Plan& p, double coef) {
-        const double* base = ring.template box<double>(seq, 0) + a.xoff;
+        const double* base = reinterpret_cast<const double*>(stage) + a.xoff;
         int4* out = sm.limbs + slot * C::SLOT;
         const int eh = kLimbExp + kLimbStep * z;
         bool ok = true;
@@ -229,7 +274,7 @@ struct F64K {
             top = min(top, depth);
             out[dst] = make_int4(v.h, v.m, v.l, 0);
         }
-        if (__any_sync(0xffffffffu, top < kLimbStep) && (tid & 31) == 0) sm.big[slot] = (unsigned)seq;
+        if (__any_sync(0xffffffffu, top < kLimbStep) && (tid & 31) == 0) sm.big[slot] = tag;
         const int n = tid - 128;
         if ((unsigned)n < 4u) {
             // w's limbs count 2^delta of u's
@@ -443,29 +488,30 @@ struct F64K {
     }
 
     // One tile (bx, by) of domain `a`, output levels kb..ke-1 (a chunk of the
-    // column; it reads one level below and one above). `seq` is the CTA's
-    // running load count; loads are numbered relative to the lowest level
-    // read, lo. Returns false if a bounded wait expired (status set, copies
-    // drained). args: `a` in memory.
+    // column; it reads one level below and one above), its first levels issued by
+    // start_tile. Loads are numbered relative to the lowest level read, lo: 0 and
+    // 1 come through the start barriers, the others through the ring. Returns
+    // false if a bounded wait expired (status set, copies drained). args: `a` in
+    // memory.
     template <bool kEq, bool kSameT>
     static __device__ bool tile_impl(Ring<Shape>& ring, const Smem& sm, const CUtensorMap* mu, const CUtensorMap* mv,
                                      const CUtensorMap* mw, const FwdArgs& a, const FwdArgs* args, const Domain& dom,
-                                     int bx, int by, int kb, int ke, long long& seq, int tid, const Plan& plan) {
-        constexpr int S = C::S;
+                                     int bx, int by, int kb, int ke, Counts& count, int tid, const Plan& plan) {
         const int tx = tid % C::TX, ty = tid / C::TX;
         const int x0 = bx * C::TX, y0 = by * C::TY;
         const int i = x0 + 1 + tx, j = y0 + 1 + ty;  // the thread's first point; the others ROWS rows up each
         const int act = i <= a.nx && j <= a.ny ? min(C::PTS, (a.ny - j) / C::ROWS + 1) : 0;  // points inside the domain
         const int nz = a.nz;
-        const int lo = kb > 0 ? kb - 1 : 0, hi = ke < nz ? ke : nz - 1;
+        const int lo = lowest(kb), hi = highest(a, ke);
         const int nl = hi - lo + 1;  // levels read
-        const long long s0 = seq;
-
-        int issued = 0;  // relative loads issued (thread 0)
-        if (tid == 0) {
-            fence_proxy_async_smem();
-            for (; issued < S && issued < nl; ++issued) ring.issue((long long)(unsigned)(s0 + issued), lo + issued, mu, mv, mw, x0, y0);
-        }
+        int issued = min(nl, 3);     // relative loads issued (thread 0)
+        auto ring_load = [&](int r) { return (long long)(unsigned)(count.ring + (r - 2)); };
+        auto wait = [&](int r) {
+            return r == 0   ? mbar_wait_bounded(&ring.full[1], count.phase1 & 1)
+                   : r == 1 ? mbar_wait_bounded(&ring.full[2], count.phase2 & 1)
+                            : ring.wait(ring_load(r));
+        };
+        auto stage = [&](int r) { return ring.base + (r == 0 ? C::RAW1 : r == 1 ? C::RAW2 : 0); };
         double* __restrict__ su = static_cast<double*>(a.su);
         double* __restrict__ sv = static_cast<double*>(a.sv);
         double* __restrict__ sw = static_cast<double*>(a.sw);
@@ -491,9 +537,8 @@ struct F64K {
         // The level split at relative level r (ok: no value refused by this
         // thread), after the CTA's barrier: its scale, kZero or kNone.
         auto settle = [&](int r, bool refused) {
-            const unsigned seq_r = (unsigned)(s0 + r);
-            if (!refused && sm.big[r % 3] == seq_r) return z;
-            const int t = rescale_level(ring.template box<double>((long long)seq_r, 0) + a.xoff, sm.limbs + (r % 3) * C::SLOT,
+            if (!refused && sm.big[r % 3] == (unsigned)(count.levels + r)) return z;
+            const int t = rescale_level(reinterpret_cast<const double*>(stage(r)) + a.xoff, sm.limbs + (r % 3) * C::SLOT,
                                         sm.range, z, dom.delta, tid);
             if (t < kNone) z = t;
             return t;
@@ -505,16 +550,16 @@ struct F64K {
 #pragma unroll
         for (int r = 0; r < 3; ++r) {
             if (r < nl && !abort) {
-                const long long q = (long long)(unsigned)(s0 + r);
-                bad |= !ring.wait(q);
-                const bool ok = split_level(ring, sm, q, lo + r, r, z, a, dom.delta, tid, plan, c_pre);
+                bad |= !wait(r);
+                const bool ok = split_level(stage(r), sm, (unsigned)(count.levels + r), lo + r, r, z, a, dom.delta, tid,
+                                            plan, c_pre);
                 if (lo + r + 1 <= hi) c_pre = coef_for(a, lo + r + 1, tid);
                 const bool refused = __syncthreads_or(bad || !ok) != 0;
                 if (refused) abort = __syncthreads_or(bad);
                 if (!abort) t[r] = settle(r, refused);
-                if (!abort && tid == 0 && issued < nl) {  // load r's stage is free again
+                if (r == 2 && !abort && tid == 0 && issued < nl) {  // the stage is free again
                     fence_proxy_async_smem();
-                    ring.issue((long long)(unsigned)(s0 + issued), lo + issued, mu, mv, mw, x0, y0);
+                    ring.issue(ring_load(issued), lo + issued, mu, mv, mw, x0, y0);
                     ++issued;
                 }
             }
@@ -567,10 +612,11 @@ struct F64K {
             t2 = kNone;
             __syncthreads();  // level k-1's limbs are free
             if (r + 2 < nl) {
-                const long long next = (long long)(unsigned)(s0 + r + 2);
-                bad |= !ring.wait(next);
+                bad |= !ring.wait(ring_load(r + 2));
                 bool ok = true;
-                if (dom.limbs) ok = split_level(ring, sm, next, k + 2, sl, z, a, dom.delta, tid, plan, c_pre);
+                if (dom.limbs)
+                    ok = split_level(ring.base, sm, (unsigned)(count.levels + r + 2), k + 2, sl, z, a, dom.delta, tid, plan,
+                                     c_pre);
                 if (k + 3 <= hi) c_pre = coef_for(a, k + 3, tid);
                 // publishes level k+2's limbs, frees its stage
                 const bool refused = __syncthreads_or(bad || !ok) != 0;
@@ -578,7 +624,7 @@ struct F64K {
                 if (!abort && dom.limbs) t2 = settle(r + 2, refused);
                 if (!abort && tid == 0 && issued < nl) {
                     fence_proxy_async_smem();
-                    ring.issue((long long)(unsigned)(s0 + issued), lo + issued, mu, mv, mw, x0, y0);
+                    ring.issue(ring_load(issued), lo + issued, mu, mv, mw, x0, y0);
                     ++issued;
                 }
             }
@@ -597,22 +643,27 @@ struct F64K {
         if (abort) {
             if (tid == 0) {
                 atomicOr(&tu_status, kStatusTimeout);
-                for (int q = (issued > S ? issued - S : 0); q < issued; ++q) (void)ring.wait((long long)(unsigned)(s0 + q));
+                for (int q = 0; q < issued; ++q)
+                    if (q < 2 || q == issued - 1) (void)wait(q);
             }
             return false;
         }
         __syncthreads();  // every read of this tile's stages and limbs is done before the next tile's
-        seq = s0 + nl;
+        count.levels += nl;
+        count.ring += max(nl - 2, 0);
+        count.phase1 += 1;
+        count.phase2 += nl > 1 ? 1 : 0;
         return true;
     }
 
     template <bool kSameT>
     static __device__ bool tile(Ring<Shape>& ring, const Smem& sm, const CUtensorMap* mu, const CUtensorMap* mv,
                                 const CUtensorMap* mw, const FwdArgs& a, const FwdArgs* args, int bx, int by, int kb,
-                                int ke, long long& seq, int tid, const Plan& plan) {
+                                int ke, Counts& count, int tid, const Plan& plan) {
+        if (tid == 0) start_tile(ring, mu, mv, mw, a, bx, by, kb, ke, count);  // (the scan runs while they arrive)
         const Domain d = scan_coefs(a, sm, tid);
-        if (d.equal) return tile_impl<true, kSameT>(ring, sm, mu, mv, mw, a, args, d, bx, by, kb, ke, seq, tid, plan);
-        return tile_impl<false, kSameT>(ring, sm, mu, mv, mw, a, args, d, bx, by, kb, ke, seq, tid, plan);
+        if (d.equal) return tile_impl<true, kSameT>(ring, sm, mu, mv, mw, a, args, d, bx, by, kb, ke, count, tid, plan);
+        return tile_impl<false, kSameT>(ring, sm, mu, mv, mw, a, args, d, bx, by, kb, ke, count, tid, plan);
     }
 };
 
@@ -632,15 +683,16 @@ __global__ void __launch_bounds__(C::NT, C::MINB) fwd_f64_kernel(const __grid_co
         prefetch_tensormap(&mu);
         prefetch_tensormap(&mv);
         prefetch_tensormap(&mw);
-        ring.init_barriers();
+        K::init_barriers(ring);
     }
     if (tid < 4) sm.big[tid] = ~0u;
     __syncthreads();
-    long long seq = 0;
+    typename K::Counts count;
     int bx, by, k0, k1;
     sched_item(sched, a.kend - a.kbeg, blockIdx.x, &bx, &by, &k0, &k1);
     const typename K::Plan plan = K::make_plan(tid);
-    (void)K::template tile<kSameT>(ring, sm, &mu, &mv, &mw, a, &a, bx, by, a.kbeg + k0, a.kbeg + k1, seq, tid, plan);
+    (void)K::template tile<kSameT>(ring, sm, &mu, &mv, &mw, a, &a, bx, by, a.kbeg + k0, a.kbeg + k1, count, tid,
+                                 plan);
 }
 
 // Persistent form over a batch plan: work items (one tile column of one
@@ -657,12 +709,12 @@ __global__ void __launch_bounds__(C::NT, C::MINB) fwd_f64_batched(BatchPlan* pla
         if (tid == 0) atomicOr(&tu_status, kStatusBadPlan);
         return;
     }
-    if (tid == 0) ring.init_barriers();
+    if (tid == 0) K::init_barriers(ring);
     if (tid < 4) sm.big[tid] = ~0u;
     __syncthreads();
     const long long n_items = plan->n_items;
     const typename K::Plan split = K::make_plan(tid);
-    long long seq = 0;
+    typename K::Counts count;
     for (long long it = 0; it < n_items; ++it) {
         if (tid == 0) *sm.item = (long long)atomicAdd(&plan->counter, 1ull);
         __syncthreads();
@@ -680,10 +732,9 @@ __global__ void __launch_bounds__(C::NT, C::MINB) fwd_f64_batched(BatchPlan* pla
         const int kb = (int)((long long)args.nz * ch / kchunks);
         const int ke = (int)((long long)args.nz * (ch + 1) / kchunks);
         const int bx = tt % tiles_x, by = tt / tiles_x;
-        const bool go = args.same_t ? K::template tile<true>(ring, sm, &d.mu, &d.mv, &d.mw, args, &d.args, bx, by, kb, ke,
-                                                             seq, tid, split)
-                                    : K::template tile<false>(ring, sm, &d.mu, &d.mv, &d.mw, args, &d.args, bx, by, kb,
-                                                              ke, seq, tid, split);
+        const bool go = args.same_t
+                            ? K::template tile<true>(ring, sm, &d.mu, &d.mv, &d.mw, args, &d.args, bx, by, kb, ke, count, tid, split)
+                            : K::template tile<false>(ring, sm, &d.mu, &d.mv, &d.mw, args, &d.args, bx, by, kb, ke, count, tid, split);
         if (!go) break;
     }
 }
