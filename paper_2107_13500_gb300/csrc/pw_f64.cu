@@ -55,8 +55,11 @@
 // 512x512x64 without density: 1043 -> 543 us (31 GPt/s); with density 1138 -> 571
 // us; 1000x250x37 with density, tcx != tcy, unaligned: 658 -> 370 us; 128x128x64:
 // 82 -> 45 us; a batch of 20 domains: 3879 -> 2078 us. Winds of 1e3 or 1e-3 times
-// that size take 557 and 623 us. A column of FP64 steps costs about 1650 us at
-// 512x512x64, more than before.
+// that size take 557 and 623 us. A field of FP64 steps only costs about 1700 us at
+// 512x512x64, more than before; winds that cross zero to rounding on a few grid
+// lines (2^-53 beside 1: those tiles fall to FP64) 1070, a Gaussian of 40 columns'
+// width around one point 1340. Cutting values below the window instead of refusing
+// them gained nothing there (their outputs are too small for the limb sums).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
