@@ -201,21 +201,27 @@ PW_LHD int limb_clz(uint32_t x) {
 // The carried sum as a double, rounded once to nearest (a tie away from zero):
 // its value is (g3 2^116 + ...) 2^scale (scale: lambda + lambda). Integer
 // operations only: the FP64 unit, slow as it is, would make every warp of a CTA
-// queue for it at the same point. Of the sum's low bits 2^-32 units of g3
-// remain. *large: the sum reaches 2^kLimbEnough units of g3; one that does not
-// may have lost bits. 0 gives 0.
+// queue for it at the same point. Of the sum's low bits 2^-29 units of g3
+// remain, also where large products cancel to a sum below one unit. *large: the
+// sum reaches 2^kLimbEnough units of g3; one that does not may have lost bits.
+// 0 gives 0.
 PW_LHD double limb_to_double(const LimbSum& s, int scale, bool* large) {
     const uint32_t t1 = static_cast<uint32_t>(s.g3 >> 32);
     const uint32_t sg = static_cast<uint32_t>(static_cast<int>(t1) >> 31);
     // the magnitude's words (one unit of the last one less, if negative)
     const uint32_t w2 = t1 ^ sg, w1 = static_cast<uint32_t>(s.g3) ^ sg, w0 = (static_cast<uint32_t>(s.g2) << 3) ^ sg;
     const bool up = w2 == 0;
-    const uint32_t a = up ? w1 : w2, b = up ? w0 : w1, c = up ? 0u : w0;
+    uint32_t a = up ? w1 : w2, b = up ? w0 : w1, c = up ? 0u : w0, base = static_cast<uint32_t>(scale + 116 + 63 + 1022);
+    if (a == 0) {  // below one unit of g3: only w0 is left
+        a = b;
+        b = 0u;
+        base -= 32u;
+    }
     const uint32_t n = static_cast<uint32_t>(limb_clz(a));
-    *large = !up || n < 32 - kLimbEnough;
+    *large = !up || w1 >= 1u << kLimbEnough;
     const uint32_t m1 = limb_shl(b, a, n), m0 = limb_shl(c, b, n);  // top bit set
     // weight of the top bit: 2^(scale + 116 + 63 - n), 32 less if up; the bit itself adds one to the exponent field
-    const uint32_t e = static_cast<uint32_t>(scale + 116 + 63 + 1022) - (up ? 32u : 0u) - n;
+    const uint32_t e = base - (up ? 32u : 0u) - n;
     const uint64_t v = (static_cast<uint64_t>(m1 >> 11) << 32 | limb_shr(m0, m1, 11)) + ((m0 >> 10) & 1u);
     const uint32_t h = static_cast<uint32_t>(v >> 32) + (e << 20);
     return limb_words(a == 0 ? 0u : h | (sg & 0x80000000u), a == 0 ? 0u : static_cast<uint32_t>(v));

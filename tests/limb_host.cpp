@@ -1,0 +1,23 @@
+// The sums of csrc/pw_limb.cuh on the host, for tests that know the exact value.
+#include "pw_limb.cuh"
+
+// su's horizontal products of n points, p = {uw, uc, ue, us, un, vs, vse, vc, ve}
+// in a window of exponent E: the sum of q(i-1) Fx(i-1/2) - q(i+1) Fx(i+1/2) and
+// the same in y as a double, and whether it reaches kLimbEnough.
+extern "C" void limb_su_sums(int n, int E, const double* p, double* out, unsigned char* in, unsigned char* enough) {
+    for (int q = 0; q < n; ++q, p += 9) {
+        pw::Limb3 l[9];
+        in[q] = 1;
+        for (int k = 0; k < 9; ++k) in[q] &= pw::limb_split(p[k], E, &l[k]) ? 1 : 0;
+        pw::LimbSum s = pw::limb_zero();
+        pw::limb_mac(s, pw::limb_sub(l[0], l[2]), pw::limb_add(pw::limb_add(l[0], l[1]), l[2]));
+        pw::limb_mac(s, l[3], pw::limb_add(l[5], l[6]));
+        pw::limb_mac(s, l[4], pw::limb_neg_sum(l[7], l[8]));
+        pw::limb_carry(s);
+        bool large;
+        out[q] = pw::limb_to_double(s, 2 * (E - 86), &large);
+        const long long m = pw::limb_least(l[0].h - l[2].h, l[0].h + l[1].h + l[2].h) +
+                            pw::limb_least(l[3].h, l[5].h + l[6].h) + pw::limb_least(l[4].h, l[7].h + l[8].h);
+        enough[q] = large || m >= (1ll << pw::kLimbEnough);
+    }
+}
