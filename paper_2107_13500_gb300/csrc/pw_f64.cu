@@ -427,8 +427,8 @@ struct F64K {
 
     // Of the outputs in `which`, whose limb sums came out small, those that the
     // limbs do not settle: neither do the magnitudes of their horizontal
-    // products reach 2^28 units, nor are all their advected values 0 (then the
-    // output is exactly 0). U, U1: the point in the slots of levels k and k+1; e: the point's
+    // products, with their coefficients, reach 2^28 units, nor are all their
+    // advected values 0 (then the output is exactly 0). U, U1: the point in the slots of levels k and k+1; e: the point's
     // offset in the fields, on level k.
     static __device__ __noinline__ unsigned unsettled(const int4* U, const int4* U1, unsigned which, bool top,
                                                       const FwdArgs* a, size_t e) {
@@ -438,22 +438,24 @@ struct F64K {
         auto zero5 = [&](const int4* q, const int4* up) {
             return zero(q[-1]) && zero(q[1]) && zero(q[-W]) && zero(q[W]) && (top || zero(*up));
         };
-        const long long enough = 1ll << kLimbEnough;
+        // (tcx and tcy over tref multiply the products before the sum is formed)
+        const int sx = a->same_t ? 0 : limb_binades(__dmul_rn(a->tcx, a->tinv));
+        const int sy = a->same_t ? 0 : limb_binades(__dmul_rn(a->tcy, a->tinv));
         unsigned left = 0;
         if ((which & 1u) && !(__ldg(static_cast<const double*>(a->u) + e - a->sz) == 0.0 && zero5(U, U1))) {
-            const long long m = limb_least(U[-1].x - U[1].x, U[-1].x + U[0].x + U[1].x) + limb_least(U[-W].x, V[-W].x + V[1 - W].x) +
-                                limb_least(U[W].x, V[0].x + V[1].x);
-            if (m < enough) left |= 1u;
+            const long long x = limb_least(U[-1].x - U[1].x, U[-1].x + U[0].x + U[1].x);
+            const long long y = limb_least(U[-W].x, V[-W].x + V[1 - W].x) + limb_least(U[W].x, V[0].x + V[1].x);
+            if (!limb_settled(x, y, sx, sy)) left |= 1u;
         }
         if ((which & 2u) && !(__ldg(static_cast<const double*>(a->v) + e - a->sz) == 0.0 && zero5(V, V1))) {
-            const long long m = limb_least(V[-W].x - V[W].x, V[-W].x + V[0].x + V[W].x) + limb_least(V[-1].x, U[-1].x + U[W - 1].x) +
-                                limb_least(V[1].x, U[0].x + U[W].x);
-            if (m < enough) left |= 2u;
+            const long long x = limb_least(V[-1].x, U[-1].x + U[W - 1].x) + limb_least(V[1].x, U[0].x + U[W].x);
+            const long long y = limb_least(V[-W].x - V[W].x, V[-W].x + V[0].x + V[W].x);
+            if (!limb_settled(x, y, sx, sy)) left |= 2u;
         }
         if ((which & 4u) && !(__ldg(static_cast<const double*>(a->w) + e - a->sz) == 0.0 && zero5(Z, Z1))) {
-            const long long m = limb_least(Z[-1].x, U[-1].x + U1[-1].x) + limb_least(Z[1].x, U[0].x + U1[0].x) +
-                                limb_least(Z[-W].x, V[-W].x + V1[-W].x) + limb_least(Z[W].x, V[0].x + V1[0].x);
-            if (m < enough) left |= 4u;
+            const long long x = limb_least(Z[-1].x, U[-1].x + U1[-1].x) + limb_least(Z[1].x, U[0].x + U1[0].x);
+            const long long y = limb_least(Z[-W].x, V[-W].x + V1[-W].x) + limb_least(Z[W].x, V[0].x + V1[0].x);
+            if (!limb_settled(x, y, sx, sy)) left |= 4u;
         }
         return left;
     }

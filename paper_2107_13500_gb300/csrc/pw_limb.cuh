@@ -234,4 +234,17 @@ PW_LHD long long limb_least(int a, int b) {
     return x > 0 && y > 0 ? limb_mul(x, y) : 0;
 }
 
+// Binades that |r| lies below 1 (|r| <= 1), rounded up; 63 for 0: products with
+// the coefficient r count at least 2^-that of their magnitude.
+PW_LHD int limb_binades(double r) {
+    const int e = static_cast<int>(limb_hi(r) >> 20 & 0x7FFu);
+    return e <= 1023 - 63 ? 63 : e >= 1023 ? 0 : 1023 - e;
+}
+
+// Whether horizontal products of magnitudes x and y (limb_least, before their
+// coefficients, which lie sx and sy binades below 1) reach 2^kLimbEnough units.
+PW_LHD bool limb_settled(long long x, long long y, int sx, int sy) {
+    return (x >> sx) + (y >> sy) >= (1ll << kLimbEnough);
+}
+
 }  // namespace pw

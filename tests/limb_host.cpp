@@ -21,3 +21,30 @@ extern "C" void limb_su_sums(int n, int E, const double* p, double* out, unsigne
         enough[q] = large || m >= (1ll << pw::kLimbEnough);
     }
 }
+
+// The same with coefficients of the x and y sums (|rx|, |ry| <= 1) as where tcx
+// and tcy differ: rx X + ry Y, and whether the sum or the magnitudes of its
+// products settle it.
+extern "C" void limb_su_joined(int n, int E, double rx, double ry, const double* p, double* out, unsigned char* in,
+                               unsigned char* enough) {
+    pw::Limb3 cx, cy;
+    (void)pw::limb_split<31>(rx, 2, &cx);
+    (void)pw::limb_split<31>(ry, 2, &cy);
+    for (int q = 0; q < n; ++q, p += 9) {
+        pw::Limb3 l[9];
+        in[q] = 1;
+        for (int k = 0; k < 9; ++k) in[q] &= pw::limb_split(p[k], E, &l[k]) ? 1 : 0;
+        pw::LimbSum x = pw::limb_zero(), y = pw::limb_zero(), s = pw::limb_zero();
+        pw::limb_mac(x, pw::limb_sub(l[0], l[2]), pw::limb_add(pw::limb_add(l[0], l[1]), l[2]));
+        pw::limb_mac(y, l[3], pw::limb_add(l[5], l[6]));
+        pw::limb_mac(y, l[4], pw::limb_neg_sum(l[7], l[8]));
+        pw::limb_mac_scaled(s, x, cx);
+        pw::limb_mac_scaled(s, y, cy);
+        pw::limb_carry(s);
+        bool large;
+        out[q] = pw::limb_to_double(s, 2 * (E - 86), &large);
+        const long long mx = pw::limb_least(l[0].h - l[2].h, l[0].h + l[1].h + l[2].h);
+        const long long my = pw::limb_least(l[3].h, l[5].h + l[6].h) + pw::limb_least(l[4].h, l[7].h + l[8].h);
+        enough[q] = large || pw::limb_settled(mx, my, pw::limb_binades(rx), pw::limb_binades(ry));
+    }
+}

@@ -55,3 +55,31 @@ def test_near_uniform_winds_keep_their_tendency(lib, wind, eps):
         a = abs(uw * (uw + uc)) + abs(ue * (uc + ue)) + abs(us * (vs + vse)) + abs(un * (vc + ve))
         err = abs(int(math.ldexp(float(got), 280)) - exact)
         assert err <= 0.5 * _ulp(exact, 280) + 2.0 ** -52 * a, (wind, eps, err / a)
+
+
+@pytest.mark.parametrize("ratio", [0.0, 1e-6, 1e-4, 0.25, 1.0 - 2.0 ** -53])
+@pytest.mark.parametrize("swap", [False, True])
+@pytest.mark.parametrize("u_scale", [1.0, 1e-4, 2.0 ** -16, 2.0 ** -19])
+def test_products_with_small_coefficients_do_not_settle_a_sum(lib, ratio, swap, u_scale):
+    """tcx != tcy: large products of the direction whose coefficient is small or
+    0 say nothing about the sum. What the rule settles is within the bound
+    above, with the coefficients in the magnitudes."""
+    n, E = 1000, 7
+    r = np.random.default_rng(5)
+    p = r.uniform(5.0, 15.0, (n, 9)) * r.choice([-1.0, 1.0], (n, 9))
+    p[:, :5] *= u_scale / 10.0
+    rx, ry = (ratio, 1.0) if swap else (1.0, ratio)
+    out, ok, enough = np.zeros(n), np.zeros(n, np.uint8), np.zeros(n, np.uint8)
+    c = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    lib.limb_su_joined(n, E, ctypes.c_double(rx), ctypes.c_double(ry), c(np.ascontiguousarray(p)), c(out), c(ok), c(enough))
+    assert ok.all()
+    cx, cy = _ints((rx, ry), 80)
+    for row, got, settled in zip(p, out, enough):
+        uw, uc, ue, us, un, vs, vse, vc, ve = _ints(row)
+        exact = cx * (uw * (uw + uc) - ue * (uc + ue)) + cy * (us * (vs + vse) - un * (vc + ve))
+        a = cx * (abs(uw * (uw + uc)) + abs(ue * (uc + ue))) + cy * (abs(us * (vs + vse)) + abs(un * (vc + ve)))
+        err = abs(int(math.ldexp(float(got), 360)) - exact)
+        if settled:
+            assert err <= 0.5 * _ulp(exact, 360) + 2.0 ** -52 * a, err / a
+    if u_scale == 1.0 and ratio > 0.1:
+        assert enough.mean() > 0.99
