@@ -427,7 +427,8 @@ __global__ void __launch_bounds__(Cfg::NT, kFull ? Cfg::MIN_BLOCKS_FULL : Cfg::M
     SplitRing<Cfg> ring;
     ring.setup(smem_raw);
     const int tid = threadIdx.x;
-    if (plan->variant != variant || (plan->dtype != PW_F32 && plan->dtype != PW_F32_SPLIT)) {
+    // the two dtypes run different arithmetic: a plan of one is no plan of the other
+    if (plan->variant != variant || plan->dtype != (kFull ? PW_F32 : PW_F32_SPLIT)) {
         if (tid == 0) atomicOr(&tu_status, kStatusBadPlan);
         return;
     }
