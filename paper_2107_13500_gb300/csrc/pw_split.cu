@@ -308,12 +308,13 @@ __device__ bool split_tile(SplitRing<Cfg, kLowBits>& ring, const CUtensorMap* mu
             }
         } else {
             // PW_F32: of the row only the coefficients are read (every operation
-            // rounds as with means of 0 in the form above, so the results are
-            // the same bits). Leaving the
-            // products with the means (all 0) out took the 512x512x64 call from
-            // 84 to 74 us (5.4 TB/s, 0.80 of the copy rate) on the same 20
-            // warps per SM, and a batch of 20 domains from 349 to 283 us, where
-            // the persistent kernel now also fits 20 warps instead of 16
+            // rounds as with means of 0 in the form above, so finite values
+            // give the same bits; 0 times an infinity is NaN there and left out
+            // here). Leaving the products with the means (all 0) out took the
+            // 512x512x64 call from 84 to 74 us (5.4 TB/s, 0.80 of the copy
+            // rate) on the same 20 warps per SM, and a batch of 20 domains from
+            // 349 to 283 us, where the persistent kernel now also fits 20 warps
+            // instead of 16
             const float zc1 = T4[1].x, zc2 = T4[1].w, zd1 = T4[5].x, zd2 = T4[5].w;
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
