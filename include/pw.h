@@ -119,11 +119,10 @@ int pw_fill_periodic_halo(pw_dtype dtype, void *field, const pw_dims *dims, void
  *   of |c||q||a+b| (the absolute values of the products the formula adds);
  *   M = the same with |a|+|b| in place of |a+b| (M >= A).
  *   PW_F64 (forward): sums of products in 87-bit fixed point, split from the
- *   doubles without error, each output rounded to double once and multiplied
- *   by the larger of tcx and tcy; values that the fixed point cannot hold
- *   beside their neighbours, infinities and NaN make the outputs that read
- *   them, or their neighbours, native FP64 evaluations term by term. Its error
- *   is a few units of 2^-53 of M, within 1e-13 of A.
+ *   doubles, each output rounded to double once and multiplied by the larger of
+ *   tcx and tcy. Outputs whose products are all far below the largest of their
+ *   neighbourhood, and those near infinities and NaN, are native FP64 evaluations
+ *   term by term. Its error is a few units of 2^-53 of M, within 1e-13 of A.
  *   PW_F64_PAIRED carries every value as an unevaluated sum of two floats
  *   (about 48 significant bits); each double is split into a pair before
  *   a + b is formed, so its error is bounded by M: within 1e-13 of M at

@@ -10,19 +10,19 @@
 //
 // A value x = (h 2^58 + m 2^29 + l) 2^lambda: h signed, m and l in [0, 2^29).
 // With |x| < 2^E, lambda = E - 86, |h| < 2^28. The split of a double is
-// exact for 0 and for every magnitude in the window [2^(E-32), 2^E); any other
-// value (subnormals, infinities and NaN included) is refused, and the caller
-// evaluates in FP64 wherever such a value takes part. Sums of up to three limb
+// exact for 0 and for every magnitude in the window [2^(E-32), 2^E); smaller
+// values are cut to the window's unit (limb_split_cut). Sums of up to three limb
 // values need no carries: their limbs stay below 2^31.
 //
 // A product keeps the limb products down to h l and m m (six of the nine), in
 // three 64-bit sums; m l and l l are dropped. A sum of six products with its
 // scaling is then within 2^-24 units of its upper sum g3 (2^-26 in practice)
-// of the exact one, and it is rounded to 53 bits once, at the end (to_double).
+// of the exact one, cut values included, and it is rounded to 53 bits once, at
+// the end (to_double).
 // So wherever the sum itself, or the sum of its products' magnitudes, reaches
 // 2^28 units of g3 (kLimbEnough), the result is closer to the exact one than
 // FP64 arithmetic, which rounds at every operation, would come. Products of
-// values in the top 12 binades of the window are 2^32 .. 2^57 units; sums whose
+// values in the top binade of the window are 2^54 .. 2^57 units; sums whose
 // products are all smaller than 2^28 are left to the caller, who evaluates them
 // in FP64.
 //
@@ -43,12 +43,10 @@ namespace pw {
 
 constexpr int kLimb = 29;
 constexpr int kLimbMask = (1 << kLimb) - 1;
-// Exponent E of the window of u and v at scale z: 7 + 12 z. A level whose
-// largest magnitude lies in [2^(E-12), 2^E) takes scale z, so that it keeps at
-// least 20 binades below it; winds of 0.03 .. 128 m/s have z = 0. The scale
-// depends on the level's own values only, and every arithmetic step on the
-// scale only, never on the launch.
-constexpr int kLimbExp = 7, kLimbStep = 12;
+// A window's exponent E is that of the largest magnitude it has to hold, so
+// fields times a power of two give the same bits, scaled. kLimbExp: where there
+// is none.
+constexpr int kLimbExp = 7;
 constexpr int kLimbWindow = 32;
 constexpr int kLimbEnough = 28;
 
@@ -133,15 +131,15 @@ PW_LHD void limb_fma(long long& s, int a, int b) {
 // window's top (negative above it, large for 0).
 template <int kTop = 28>
 PW_LHD bool limb_split(double x, int E, Limb3* out, int* depth = nullptr) {
-    const uint32_t hi = limb_hi(x), lo = limb_lo(x);
-    const uint32_t e = hi & 0x7FF00000u;
+    const uint32_t hi = limb_hi(x), lo = limb_lo(x), mag = hi & 0x7FFFFFFFu;
     // the implicit bit, absent from zero (and from subnormals, refused below)
-    const uint32_t mh = (hi & 0x000FFFFFu) | (e < 0x00100000u ? e : 0x00100000u);
+    const uint32_t one = mag < 0x00100000u ? mag : 0x00100000u;
+    const uint32_t mh = (hi & 0x000FFFFFu) | (one & 0xFFF00000u);
     // significand with its top bit at bit kTop - 1 of the upper word, then the shift that aligns it
     const uint32_t a1 = limb_shl(lo, mh, kTop - 21), a0 = lo << (kTop - 21);
-    const int d = static_cast<int>((static_cast<uint32_t>(E - 1 + 1023) << 20) - e) >> 20;
+    const int d = static_cast<int>((static_cast<uint32_t>(E - 1 + 1023) << 20 | 0xFFFFFu) - mag) >> 20;
     if (depth) *depth = d;
-    const bool ok = static_cast<uint32_t>(d) < static_cast<uint32_t>(kLimbWindow) || (mh | lo) == 0;
+    const bool ok = static_cast<uint32_t>(d) < static_cast<uint32_t>(kLimbWindow) || (mag | lo) == 0;
     const uint32_t s = static_cast<uint32_t>(static_cast<int>(hi) >> 31);
     const uint64_t sn = (static_cast<uint64_t>(s) << 32) | s;
     const uint64_t n = (((static_cast<uint64_t>(a1) << 32) | a0) ^ sn) - sn;  // with the sign
@@ -152,6 +150,85 @@ PW_LHD bool limb_split(double x, int E, Limb3* out, int* depth = nullptr) {
     out->m = static_cast<int>(w1 >> 3);
     out->l = static_cast<int>(limb_shr(w0, w1, 6) & static_cast<uint32_t>(kLimbMask));
     return ok;
+}
+
+// Magnitude words x2 2^64 + x1 2^32 + x0, whose bit 6 is the limbs' unit, shifted
+// down by s (0 .. 95; up by -s where s < 0, -95 at most) and cut there, as signed
+// limbs. *cut: something was lost.
+PW_LHD Limb3 limb_place(uint32_t x2, uint32_t x1, uint32_t x0, int s, bool negative, bool* cut) {
+    uint32_t lost = 0;
+    if (s < 0) {
+        const uint32_t t = static_cast<uint32_t>(-s);
+        if (t >= 64) x2 = x0, x1 = x0 = 0;
+        else if (t >= 32) x2 = x1, x1 = x0, x0 = 0;
+        x2 = limb_shl(x1, x2, t), x1 = limb_shl(x0, x1, t), x0 <<= t & 31u;
+    } else {
+        const uint32_t t = static_cast<uint32_t>(s);
+        if (t >= 64) lost = x1 | x0, x0 = x2, x1 = x2 = 0;
+        else if (t >= 32) lost = x0, x0 = x1, x1 = x2, x2 = 0;
+        lost |= limb_shr(0u, x0, t);  // the bits below x0
+        x0 = limb_shr(x0, x1, t), x1 = limb_shr(x1, x2, t), x2 >>= t & 31u;
+    }
+    *cut = (lost | (x0 & 63u)) != 0;
+    uint64_t low = (static_cast<uint64_t>(x1) << 32 | x0) >> 6;  // m and l
+    int h = static_cast<int>(x2);
+    if (negative) {
+        h = low != 0 ? ~h : -h;
+        low = (0 - low) & ((1ull << 58) - 1);
+    }
+    return {h, static_cast<int>(low >> kLimb), static_cast<int>(low) & kLimbMask};
+}
+
+// The split for a value below the window (its top bit 32 binades or more under
+// 2^E), cut towards zero to the unit, 2^(E - 86): off by less than that, which
+// moves a product by less than 2^-28 units of g3. Returns whether anything was cut.
+PW_LHD bool limb_split_low(double x, int E, Limb3* out) {
+    const uint32_t hi = limb_hi(x), lo = limb_lo(x), e = hi >> 20 & 0x7FFu;
+    const uint32_t mh = (hi & 0x000FFFFFu) | (e ? 0x00100000u : 0u);
+    const uint32_t a1 = limb_shl(lo, mh, 7), a0 = lo << 7;  // as in limb_split
+    const int d = E - 1 + 1023 - static_cast<int>(e ? e : 1u);
+    const uint32_t s = static_cast<uint32_t>(d > 95 ? 95 : d), x1 = s < 64 ? a1 : 0u, x0 = s < 64 ? a0 : a1;
+    const uint32_t y0 = limb_shr(x0, x1, s), y1 = x1 >> (s & 31u);
+    const uint32_t lost = (s < 64 ? 0u : a0) | limb_shr(0u, x0, s) | (y0 & 63u);
+    uint64_t low = (static_cast<uint64_t>(y1) << 32 | y0) >> 6;
+    const bool minus = static_cast<int>(hi) < 0 && low != 0;
+    if (minus) low = (1ull << 58) - low;
+    *out = {minus ? -1 : 0, static_cast<int>(low >> kLimb), static_cast<int>(low) & kLimbMask};
+    return lost != 0;
+}
+
+// The split for any |x| < 2^E, cut like that where it lies below the window; the
+// unit is 2^-87 for kTop = 31, E = 2.
+template <int kTop = 28>
+PW_LHD bool limb_split_cut(double x, int E, Limb3* out) {
+    const uint32_t hi = limb_hi(x), lo = limb_lo(x), e = hi >> 20 & 0x7FFu;
+    const uint32_t mh = (hi & 0x000FFFFFu) | (e ? 0x00100000u : 0u);
+    const int d = E - 1 + 1023 - static_cast<int>(e ? e : 1u);
+    bool cut;
+    *out = limb_place(limb_shl(lo, mh, kTop - 21), lo << (kTop - 21), 0u, d < 0 ? 0 : d > 95 ? 95 : d, hi >> 31 != 0, &cut);
+    return cut;
+}
+
+// The limbs of a value in a window whose exponent is up larger (95 either way at
+// most), as limb_split_cut would have them.
+PW_LHD Limb3 limb_shift(Limb3 a, int up, bool* cut) {
+    uint64_t low = static_cast<uint64_t>(a.m) << kLimb | static_cast<uint32_t>(a.l);
+    if (up > -32 && up < 32) {  // where nothing is cut, the words shift with their sign
+        const uint32_t x2 = static_cast<uint32_t>(a.h), x1 = static_cast<uint32_t>(low >> 26), x0 = static_cast<uint32_t>(low << 6);
+        const uint32_t s = static_cast<uint32_t>(up < 0 ? -up : up);
+        const uint32_t y0 = up < 0 ? x0 << s : limb_shr(x0, x1, s), y1 = up < 0 ? limb_shl(x0, x1, s) : limb_shr(x1, x2, s);
+        const int h = up < 0 ? static_cast<int>(limb_shl(x1, x2, s)) : a.h >> s;
+        *cut = false;
+        if (up < 0 || (limb_shr(0u, x0, s) | (y0 & 63u)) == 0)
+            return {h, static_cast<int>(y1 >> 3), static_cast<int>(limb_shr(y0, y1, 6) & static_cast<uint32_t>(kLimbMask))};
+    }
+    int h = a.h;
+    if (h < 0) {
+        h = low != 0 ? ~h : -h;
+        low = (0 - low) & ((1ull << 58) - 1);
+    }
+    low <<= 6;
+    return limb_place(static_cast<uint32_t>(h), static_cast<uint32_t>(low >> 32), static_cast<uint32_t>(low), up, a.h < 0, cut);
 }
 
 PW_LHD Limb3 limb_add(Limb3 a, Limb3 b) { return {a.h + b.h, a.m + b.m, a.l + b.l}; }
@@ -201,30 +278,44 @@ PW_LHD int limb_clz(uint32_t x) {
 // The carried sum as a double, rounded once to nearest (a tie away from zero):
 // its value is (g3 2^116 + ...) 2^scale (scale: lambda + lambda). Integer
 // operations only: the FP64 unit, slow as it is, would make every warp of a CTA
-// queue for it at the same point. Of the sum's low bits 2^-29 units of g3
-// remain, also where large products cancel to a sum below one unit. *large: the
-// sum reaches 2^kLimbEnough units of g3; one that does not may have lost bits.
-// 0 gives 0.
-PW_LHD double limb_to_double(const LimbSum& s, int scale, bool* large) {
+// queue for it at the same point. *mag: the upper word of the result's magnitude
+// (limb_small). A sum below one unit of g3 gives 0: products that cancel that far
+// are for limb_tiny.
+PW_LHD double limb_to_double(const LimbSum& s, int scale, uint32_t* mag) {
     const uint32_t t1 = static_cast<uint32_t>(s.g3 >> 32);
     const uint32_t sg = static_cast<uint32_t>(static_cast<int>(t1) >> 31);
     // the magnitude's words (one unit of the last one less, if negative)
     const uint32_t w2 = t1 ^ sg, w1 = static_cast<uint32_t>(s.g3) ^ sg, w0 = (static_cast<uint32_t>(s.g2) << 3) ^ sg;
     const bool up = w2 == 0;
-    uint32_t a = up ? w1 : w2, b = up ? w0 : w1, c = up ? 0u : w0, base = static_cast<uint32_t>(scale + 116 + 63 + 1022);
-    if (a == 0) {  // below one unit of g3: only w0 is left
-        a = b;
-        b = 0u;
-        base -= 32u;
-    }
+    const uint32_t a = up ? w1 : w2, b = up ? w0 : w1, c = up ? 0u : w0;
     const uint32_t n = static_cast<uint32_t>(limb_clz(a));
-    *large = !up || w1 >= 1u << kLimbEnough;
     const uint32_t m1 = limb_shl(b, a, n), m0 = limb_shl(c, b, n);  // top bit set
     // weight of the top bit: 2^(scale + 116 + 63 - n), 32 less if up; the bit itself adds one to the exponent field
-    const uint32_t e = base - (up ? 32u : 0u) - n;
+    const uint32_t e = static_cast<uint32_t>(scale + 116 + 63 + 1022) - (up ? 32u : 0u) - n;
     const uint64_t v = (static_cast<uint64_t>(m1 >> 11) << 32 | limb_shr(m0, m1, 11)) + ((m0 >> 10) & 1u);
-    const uint32_t h = static_cast<uint32_t>(v >> 32) + (e << 20);
-    return limb_words(a == 0 ? 0u : h | (sg & 0x80000000u), a == 0 ? 0u : static_cast<uint32_t>(v));
+    const uint32_t h = a == 0 ? 0u : static_cast<uint32_t>(v >> 32) + (e << 20);
+    *mag = h;
+    return limb_words(h | (sg & 0x80000000u), a == 0 ? 0u : static_cast<uint32_t>(v));
+}
+
+// Whether a result of that upper word is less than 2^kLimbEnough units of g3: one
+// that may have lost bits.
+PW_LHD bool limb_small(uint32_t mag, int scale) {
+    return mag < static_cast<uint32_t>(scale + 116 + kLimbEnough + 1023) << 20;
+}
+
+PW_LHD double limb_to_double(const LimbSum& s, int scale, bool* large) {
+    uint32_t mag;
+    const double x = limb_to_double(s, scale, &mag);
+    *large = !limb_small(mag, scale);
+    return x;
+}
+
+// A carried sum that limb_to_double gave as 0, from what is left of it: 2^-29
+// units of g3.
+PW_LHD double limb_tiny(const LimbSum& s, int scale) {
+    const int t = static_cast<int>(static_cast<uint32_t>(s.g3) << kLimb | (static_cast<uint32_t>(s.g2) & kLimbMask));
+    return static_cast<double>(t) * limb_words(static_cast<uint32_t>(scale + 116 - kLimb + 1023) << 20, 0u);
 }
 
 // A lower bound of |a b| in units of g3 from the upper limbs of a and b, sums of
