@@ -29,7 +29,7 @@
 // left most points of winds over dx >= 20 dz to FP64.) Values below their window
 // are cut to its unit; an output whose products are all too small for the limb
 // sums (kLimbEnough) is evaluated in FP64, term by term, from a list that the CTA
-// works off with whole warps. Steps that read an infinity or a NaN, or a domain
+// works off with whole warps beside the next step's points. Steps that read an infinity or a NaN, or a domain
 // whose coefficients no limb number holds, are evaluated in FP64 throughout. All
 // of that depends on the data of the tile and its levels only, not on the launch.
 //
@@ -59,15 +59,16 @@
 // largest magnitudes found in a pass of their own ahead of the first barrier cost
 // 6 % more, a decision by one warp 2 %, a top level compiled without its upper
 // face's sums from zeros in their place 2 %.
-// 512x512x64, native FP64 before -> now (us): smooth winds dx = 50 m 1066 -> 607,
-// dx = 400 1060 -> 615, dx = 4000 1060 -> 617; with density 1157 -> 638; dx = 40,
-// dy = 60 m 1062 -> 690; i.i.d. winds dx = 50 m 1062 -> 585, 1000 m 1062 -> 597;
-// w = 0 1064 -> 605; v and w of 1e-8 beside u = 5 1059 -> 785; Taylor-Green 1064
-// -> 800; sines that vanish on a grid of lines 1062 -> 1030. Slower than native
+// 512x512x64, native FP64 before -> now (us): smooth winds dx = 50 m 1066 -> 601,
+// dx = 400 1060 -> 609, dx = 4000 1060 -> 611; with density 1157 -> 635; dx = 40,
+// dy = 60 m 1062 -> 680; i.i.d. winds dx = 50 m 1062 -> 584, 1000 m 1062 -> 595;
+// w = 0 1064 -> 603; v and w of 1e-8 beside u = 5 1059 -> 765; Taylor-Green 1064
+// -> 790; sines that vanish on a grid of lines 1062 -> 980. Slower than native
 // FP64: a bump of 20 columns' width on nothing (its outskirts vary by more binades
-// in one tile than the sums hold) 1067 -> 1620, levels whose magnitudes differ by
-// 8 from each to the next 1063 -> 1290, magnitudes random over 14 decades 1062 ->
-// 1780, NaN throughout 1062 -> 1700.
+// in one tile than the sums hold) 1067 -> 1470, levels whose magnitudes differ by
+// 8 from each to the next 1063 -> 1250, magnitudes random over 14 decades 1062 ->
+// 1660, NaN throughout 1062 -> 1690. (The FP64 outputs of half the warps before
+// their points and of half after them: 1400 for the bump, but 2 % on every call.)
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -99,7 +100,7 @@ struct F64Cfg {
     static constexpr int REST = CELLS - 2 * NT, HALF = NT / 2;
     static_assert(REST > 0 && REST <= HALF, "three cells of a field per thread at most");
     // ring stages | ring barriers (64 B) | limbs [SLOTS][SLOT] | coefficients [4][4] + 2 as limbs | as doubles |
-    // scale [4] | largest magnitudes [4] | coefficient exponents [4] | item | list counts [2], [1] | lists [2] | arguments | slack
+    // scale [4] | largest magnitudes [4] | coefficient exponents [4] | item | list counts [2], [2] | lists [2] | arguments | slack
     static constexpr int LIMB_OFFSET = S * Shape::STAGE_BYTES + 64;
     static constexpr int COEF_OFFSET = LIMB_OFFSET + SLOTS * SLOT * 16;
     static constexpr int RAW_OFFSET = COEF_OFFSET + (4 * 4 + 2) * 16;
@@ -144,7 +145,7 @@ struct F64K {
         __device__ __forceinline__ int* cexp() const { return at<int>(C::EXP_OFFSET); }
         // work item handed from thread 0 to the CTA
         __device__ __forceinline__ long long* item() const { return at<long long>(C::ITEM_OFFSET); }
-        // [2]: entries of the list, by the step's parity; [2]: those of the second list
+        // [2]: entries of the list, by the step's parity; [2], [3]: those of the second list
         __device__ __forceinline__ int* count() const { return at<int>(C::ITEM_OFFSET + 8); }
         // points with outputs whose sums are small: row TX + column | these << 9 | those below one unit << 12
         __device__ __forceinline__ unsigned short* list() const { return at<unsigned short>(C::LIST_OFFSET); }
@@ -157,6 +158,15 @@ struct F64K {
     static __device__ __forceinline__ void setup(unsigned char* raw, Ring<Shape>& ring, Smem& sm) {
         ring.setup(raw);
         sm.base = ring.base;
+    }
+
+    // The same in functions of their own, found from the kernel's array so that the
+    // compiler knows their accesses as shared ones.
+    static __device__ __forceinline__ Smem here() {
+        extern __shared__ unsigned char smem_raw[];
+        Ring<Shape> ring;
+        ring.setup(smem_raw);
+        return Smem{ring.base};
     }
 
     // The ring's barrier, and one for each of a tile's first two levels.
@@ -443,8 +453,9 @@ struct F64K {
     // the new windows. Cells that were cut, and levels that exceeded their window,
     // are split again from global memory (their boxes are gone). Every thread of
     // the CTA calls it, with no limb being read.
-    static __device__ __noinline__ void rescale(Smem sm, const FwdArgs* args, int x0, int y0, int k, bool top,
+    static __device__ __noinline__ void rescale(const FwdArgs* args, int x0, int y0, int k, bool top,
                                                 int3 slots, Scale z, int tid) {
+        const Smem sm = here();
         const FwdArgs& a = *args;
         const Scale cur = scale(sm);
         for (int f = 0; f < 3; ++f) {
@@ -581,8 +592,7 @@ struct F64K {
 
     // Output f of a point in native FP64, term by term, from global memory, and its
     // store (e: the point's offset in the fields, on level k).
-    static __device__ __noinline__ void native_output(const FwdArgs* args, size_t e, int k, int f) {
-        const FwdArgs& a = *args;
+    static __device__ __forceinline__ void native_inline(const FwdArgs& a, size_t e, int k, int f) {
         const size_t sy = (size_t)a.sy, sz = (size_t)a.sz;
         const double *U = static_cast<const double*>(a.u) + e, *V = static_cast<const double*>(a.v) + e;
         const double *Wl = static_cast<const double*>(a.w) + e;
@@ -617,12 +627,15 @@ struct F64K {
         static_cast<double*>(x ? a.su : a.sv)[e] = s;
     }
 
+    static __device__ __noinline__ void native_output(const FwdArgs* args, size_t e, int k, int f) { native_inline(*args, e, k, f); }
+
     // Output f of a point in limbs once more, where the products cancel to less than
     // one unit: from the sum's lowest bits. (B, M, P: the point in the slots of levels
     // k-1, k and k+1. The general form serves all cases: on the top level the upper
     // coefficients are 0.)
-    static __device__ __noinline__ double low_output(Smem sm, const int4* B, const int4* M, const int4* P, int lev, int f,
+    static __device__ __noinline__ double low_output(const int4* B, const int4* M, const int4* P, int lev, int f,
                                                      double tref) {
+        const Smem sm = here();
         constexpr int W = C::W, N = C::CELLS;
         const Slot U{M}, V{M + N}, Z{M + 2 * N}, U1{P}, V1{P + N}, Q{M + f * N}, Q1{P + f * N}, Qb{B + f * N}, Zb{B + 2 * N};
         // twice the advecting velocities at the faces of the output's cell: lower and upper x, y, z
@@ -654,10 +667,12 @@ struct F64K {
     // The listed outputs of step k: those whose limb sums came out small. Where the
     // magnitudes of their horizontal products, with their coefficients, reach 2^28
     // units, the sum stands, from its lowest bits where it is below one unit. It is
-    // exactly 0 where all advected values are. The others are evaluated in FP64, from
-    // a list of their own so that whole warps do so.
-    static __device__ __noinline__ void listed_outputs(Smem sm, const FwdArgs* args, int listed, int x0, int y0, int k,
+    // exactly 0 where all advected values are. The others are FP64's: if they are few,
+    // at once, otherwise on a list of their own, for whole warps (late_outputs).
+    // Returns whether there is one.
+    static __device__ __noinline__ bool listed_outputs(const FwdArgs* args, int listed, int x0, int y0, int k, int* count,
                                                        int3 slots, int tid) {
+        const Smem sm = here();
         constexpr int W = C::W, N = C::CELLS;
         const FwdArgs& a = *args;
         const bool top = k == a.nz - 1;
@@ -687,29 +702,36 @@ struct F64K {
             const size_t e = (size_t)k * (size_t)a.sz + (size_t)(y0 + 1 + row) * (size_t)a.sy + (size_t)(x0 + 1 + col);
             if (limb_settled(x, y, sx, sy)) {
                 if (entry >> (12 + f) & 1u)
-                    static_cast<double*>(f == 0 ? a.su : f == 1 ? a.sv : a.sw)[e] = low_output(sm, B, U, U1, k, f, a.tref);
+                    static_cast<double*>(f == 0 ? a.su : f == 1 ? a.sv : a.sw)[e] = low_output(B, U, U1, k, f, a.tref);
             } else if (!(zero(Q[-1]) && zero(Q[1]) && zero(Q[-W]) && zero(Q[W]) && zero(B[f * N]) && (top || zero(U1[f * N])))) {
                 if (few) native_output(args, e, k, f);
-                else sm.list64()[atomicAdd(&sm.count()[2], 1)] = (unsigned short)(id | (unsigned)f << 9);
+                else sm.list64()[atomicAdd(count, 1)] = (unsigned short)(id | (unsigned)f << 9);
             }
         }
-        __syncthreads();
-        if (few) return;
-        const int left = sm.count()[2];
+        __syncthreads();  // the limbs and the list are read
+        return !few;
+    }
+
+    // The outputs of step k on the second list. They need no limbs, so they run with
+    // the next step's points: the FP64 unit works beside the integer pipes of other
+    // warps.
+    static __device__ __noinline__ void late_outputs(const FwdArgs* args, int left, int x0, int y0, int k, int tid) {
+        const Smem sm = here();
+        const FwdArgs& a = *args;
+#pragma unroll 2
         for (int q = tid; q < left; q += C::NT) {
             const int entry = sm.list64()[q], id = entry & 0x1FF;
-            native_output(args, (size_t)k * (size_t)a.sz + (size_t)(y0 + 1 + id / C::TX) * (size_t)a.sy +
-                                    (size_t)(x0 + 1 + id % C::TX), k, entry >> 9);
+            native_inline(a, (size_t)k * (size_t)a.sz + (size_t)(y0 + 1 + id / C::TX) * (size_t)a.sy +
+                                 (size_t)(x0 + 1 + id % C::TX), k, entry >> 9);
         }
-        __syncthreads();  // the limbs and the lists are read
-        if (tid == 0) sm.count()[2] = 0;
     }
 
     // Step k's windows where holds says that they are not those of the limbs: makes
     // them so. False where no windows hold the values. Every thread of the CTA calls
     // it.
-    static __device__ __noinline__ bool change_scale(Smem sm, const FwdArgs* args, int x0, int y0, int k,
+    static __device__ __noinline__ bool change_scale(const FwdArgs* args, int x0, int y0, int k,
                                                          bool top, int3 slots, int tid) {
+        const Smem sm = here();
         const int2 te = make_int2(sm.scale()[1].x, sm.scale()[1].y);
         unsigned flags;
         int base;
@@ -717,7 +739,7 @@ struct F64K {
         if (z.d == kNone) return false;
         const Scale cur = scale(sm);
         const bool same = z.u == cur.u && z.v == cur.v && z.w == cur.w && z.d == cur.d;
-        if (!same) rescale(sm, args, x0, y0, k, top, slots, z, tid);
+        if (!same) rescale(args, x0, y0, k, top, slots, z, tid);
         __syncthreads();  // (every thread has read the scale)
         if (tid == 0) store_scale(sm, z, base, flags, te);
         __syncthreads();
@@ -778,7 +800,7 @@ struct F64K {
             if (r < nl) store_coefs<false>(sm, a, lo + r, coef[r], tid);
         for (int r = 0; r < 3 && r < nl; ++r) bad |= !wait(r);
         if (tid < 4) sm.top()[tid] = make_int4(kUnset, kUnset, kUnset, 0);
-        if (tid < 3) sm.count()[tid] = 0;
+        if (tid < 4) sm.count()[tid] = 0;
         bool abort = __syncthreads_or(bad);
         if (!abort && a.limbs && nl > 1) {
             for (int r = 0; r < 3 && r < nl; ++r) scan_level(box(r), sm, lo + r, tid, plan);
@@ -804,13 +826,16 @@ struct F64K {
 
         // Level k = lo + r from the limb slots of r-1, r and r+1 (sl, sc, sp);
         // level k+2 then goes into slot sl.
+        bool late = false;  // the step before left outputs to late_outputs
         auto step = [&](auto top, int sl, int sc, int sp, int r) {
             constexpr bool kTop = decltype(top)::value;
             const int k = lo + r;
+            if (late) late_outputs(args, sm.count()[2 + ((r + 1) & 1)], x0, y0, k - 1, tid);
+            late = false;
             if (!kTop && tid == 0) sm.count()[(r + 1) & 1] = 0;  // (read in the step before)
             bool limbs = a.limbs;
             if (limbs && !holds(sm, k, kTop)) {
-                limbs = change_scale(sm, args, x0, y0, k, kTop, make_int3(sl, sc, sp), tid);
+                limbs = change_scale(args, x0, y0, k, kTop, make_int3(sl, sc, sp), tid);
             }
             const int4* B = sm.limbs() + sl * C::SLOT + c;
             const int4* M = sm.limbs() + sc * C::SLOT + c;
@@ -850,7 +875,8 @@ struct F64K {
             g += gsz;
             __syncthreads();  // level k-1's limbs are free, the list is complete
             const int listed = sm.count()[r & 1];
-            if (listed != 0) listed_outputs(sm, args, listed, x0, y0, k, make_int3(sl, sc, sp), tid);
+            if (listed != 0) late = listed_outputs(args, listed, x0, y0, k, &sm.count()[2 + (r & 1)], make_int3(sl, sc, sp), tid);
+            if (tid == 0) sm.count()[2 + ((r + 1) & 1)] = 0;  // (read at this step's start)
             if (kTop) return;
             if (r + 2 < nl) {
                 if (tid == 0) sm.top()[(k + 3) & 3] = make_int4(kUnset, kUnset, kUnset, 0);  // (level k-1's: read no more)
@@ -880,6 +906,7 @@ struct F64K {
             sp = freed;
         }
         if (ke == nz && k1 < ke && !abort) step(std::true_type(), sl, sc, sp, nz - 1 - lo);  // the domain's top level
+        if (late) late_outputs(args, sm.count()[2 + ((ke - 1 - lo) & 1)], x0, y0, ke - 1, tid);
         if (abort) {
             if (tid == 0) {
                 atomicOr(&tu_status, kStatusTimeout);
