@@ -137,7 +137,9 @@ int pw_fill_periodic_halo(pw_dtype dtype, void *field, const pw_dims *dims, void
  * dtype PW_F32: u, v, w, su, sv, sw are float full fields; `split` is the
  *   table of pw_make_split_table built with all means 0 (it then carries
  *   only the coefficients, rounded to float; nothing else of it is read).
- *   A table with means belongs to PW_F32_SPLIT, whichever fields it is for.
+ *   A table with means belongs to PW_F32_SPLIT, whichever fields it is for;
+ *   pw_device_status reports it here as PW_EINVAL (one level of each column of
+ *   tiles is looked at).
  * Errors: PW_ENULL, PW_EINVAL, PW_EALIAS, PW_EUNSUPPORTED, PW_ECUDA.
  */
 int pw_advect(pw_dtype dtype, const void *u, const void *v, const void *w, const pw_coeffs *c,
@@ -383,7 +385,8 @@ int pw_energy_budget(const void *u, const void *v, const void *w, int wind_elem_
  * current device (synchronises `stream`). *status receives 0, PW_ETIMEOUT if
  * a kernel gave up on a bounded wait since the last call, or PW_EINVAL if a
  * batched launch met a plan built for another dtype or variant (outputs of
- * those launches are unspecified). Errors: PW_ENULL, PW_ECUDA.
+ * those launches are unspecified) or a PW_F32 launch a table with level means
+ * (left out of its outputs). Errors: PW_ENULL, PW_ECUDA.
  */
 int pw_device_status(int *status, void *stream);
 

@@ -30,6 +30,10 @@ namespace {
 
 constexpr int kStrip = 4;
 constexpr int kRowBytes = PW_SPLIT_NCOEF * 4;
+// Entries of a table row that come from the means: all but tzc1, tzc2, tzd1, tzd2
+// (4, 7, 20, 23), tcx and tcy (26, 27).
+constexpr unsigned kMeanEntries = 0x03FFFFFFu & ~(1u << 4 | 1u << 7 | 1u << 20 | 1u << 23);
+static_assert(PW_SPLIT_NCOEF == 32, "a thread per entry");
 
 // Resident warps per SM the one-shot and the persistent kernels are
 // compiled for, whatever the CTA size (the register budget follows).
@@ -183,6 +187,11 @@ __device__ bool split_tile(SplitRing<Cfg, kLowBits>& ring, const CUtensorMap* mu
 
     bool bad = !ring.wait(s0);
     if (nl > 1) bad |= !ring.wait(s0 + 1);
+    // A table with means is PW_F32_SPLIT's, whose terms this march leaves out:
+    // reported. (Looked for in one row a tile column: in every row it cost 8 % of a
+    // batch, and following the general form there 120 %, by its registers.)
+    if (!kMeans && nl > 1 && !bad && tid < 32 && (kMeanEntries >> tid & 1u) != 0 && ring.row(s0 + 1)[tid] != 0.0f)
+        atomicOr(&tu_status, kStatusBadPlan);
     float uo_m[4], vo_m[4], wo_m[4], wx_m[4], wy_m[4], wz_m[4];
     {
         const float* U = ring.box(s0, 0) + cb;
