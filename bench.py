@@ -368,7 +368,7 @@ def run_only(args):
         x, means = zip(*(pw.split_field(t, nx, ny) for t in x64))
         table = torch.from_numpy(pw.make_split_table(c, *(m.cpu().numpy() for m in means))).cuda()
     elif mode == "f32":
-        x = [pw.empty_field(nx, ny, nz, torch.float32).copy_(t) for t in x64]
+        x = [pw.field_from_numpy(a, nx, torch.float32) for a in synth.fields_iid(nx, ny, nz, seed=1)]
     else:
         x = x64
     out = tuple(pw.field_like(x[0]) for _ in range(3))
