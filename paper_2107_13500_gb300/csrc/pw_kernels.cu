@@ -1,8 +1,8 @@
 // pw_kernels.cu -- helper kernels of the PW advection library: periodic halo
 // fill, the per-level mean/perturbation split, the bounded-wait self-test
-// and the device status word. The forward kernels live in pw_f64.cu (native
-// FP64), pw_paired.cu (paired FP32) and pw_split.cu (FP32); the adjoint in
-// pw_adjoint.cu.
+// and the device status word. The forward kernels live in pw_f64.cu (FP64, in
+// fixed point), pw_paired.cu (paired FP32) and pw_split.cu (FP32); the adjoint in
+// pw_adjoint.cu and pw_adjoint_f64.cu.
 #include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_runtime.h>

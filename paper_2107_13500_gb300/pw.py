@@ -322,7 +322,7 @@ def _arithmetic(mode, split_table):
 def advect(u, v, w, coeffs: Coefficients, nx, ny, mode="paired", split_table=None, out=None, stream=None):
     """Source terms (su, sv, sw) of u, v, w.
 
-    mode: "f64" (native FP64), "paired" (FP64 in/out, paired-FP32
+    mode: "f64" (FP64 accuracy), "paired" (FP64 in/out, paired-FP32
     arithmetic), "split" (float perturbations; ``split_table`` is the
     device table from :func:`make_split_table`) or "f32" (float full fields).
     """
