@@ -401,7 +401,8 @@ struct F64K {
         constexpr int kAny = 1 << 20;
         const unsigned zero = ~flags;
         const bool plain = (flags & kPlain) != 0;
-        const int other = plain ? b : max(z.u + te.x, z.v + te.y);  // beside w's, under d
+        // what holds d up beside w (a field of zeros does not)
+        const int other = max(plain || (zero & 1u) ? b : z.u + te.x, plain || (zero & 2u) ? b : z.v + te.y);
         const bool nw = (zero & 4u) == 0;
         // a field of zeros stays one; u and v of a plain scale reach its slack; others stay in their window
         auto least = [&](unsigned f, int e) { return zero & f ? -kAny : e; };
